@@ -237,14 +237,15 @@ def work(case):
 
 def tolerance(case):
     """About four times the distance from `exact` that the sums of each form show (FP32:
-    1.1e-6 at K = 4096 and 1.6e-6 at 8192; tensor cores: 4.4e-6 to 4.7e-6, whose FP32
-    accumulators do not round to nearest; training step: 1.4e-7)."""
+    1.1e-6 at K = 4096 and 1.6e-6 at 8192; tensor cores, whose FP32
+    accumulators do not round to nearest: split 4.7e-6 to 6.3e-6, BF16 and FP8 4.4e-6 and,
+    in the longest sums, 1e-5; training step: 1.4e-7)."""
     kind = case["kind"]
     if kind in ("transpose", "jacobi"):
         return "exact"
     if kind == "train":
         return {"rel": 2e-6}
-    return {"rel": 6e-6 if case["form"] == "f32" else 2e-5}
+    return {"rel": {"f32": 6e-6, "split": 2.5e-5}.get(case["form"], 4e-5)}
 
 
 def _fp8_values(x):
