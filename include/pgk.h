@@ -314,9 +314,10 @@ PGK_API pgk_status pgk_select_case_transpose(const pgk_machine* machine, const i
                                              pgk_case* out);
 
 /* dst = src^T on 32-bit words: src rows x cols (lds >= cols), dst cols x rows
- * (ldd >= rows), device pointers.  prog NULL = (B0, B1, s) = (8, 32, 2), the
- * paper's best block for order 2^14.  Errors: INVALID_ARG, INFEASIBLE,
- * UNSUPPORTED, CUDA. */
+ * (ldd >= rows), device pointers.  prog NULL = a 64 x 64 tile per block with
+ * 128-bit accesses (where the bases and row strides are multiples of 16 bytes),
+ * outside the case discussion; (8, 32, 2) is the paper's best block for order
+ * 2^14.  Errors: INVALID_ARG, INFEASIBLE, UNSUPPORTED, CUDA. */
 PGK_API pgk_status pgk_transpose(int rows, int cols, const void* src, int lds, void* dst, int ldd,
                                  const pgk_params* prog, void* stream);
 
