@@ -238,7 +238,9 @@ def summarize_k(recs, k):
 
 
 def default_index(cands, M, N, K, dtype):
-    """Index of the library's untuned default parameters in the candidate set."""
+    """Index in the candidate set of one fixed program per form (FP32: one per output
+    size), the choice without tuning or model that the evaluation compares with.  The
+    library itself plans a call without parameters by its shape."""
     if dtype == pgk.F32:
         big = M * N >= 2048 * 2048
         mid = M * N >= 256 * 256

@@ -3,8 +3,8 @@
 // The host packs the problems into a device table, ordered by decreasing K
 // (the cost of one tile), with the prefix sums of their tile counts.  Every
 // CTA repeatedly takes the next work item from an atomic counter, finds its
-// problem by binary search in the prefix sums and runs the register-blocked
-// tile (simt_rb.cuh) on it, until all tiles are handed out.  No item waits on
+// problem by a search in the prefix sums and runs the register-blocked
+// tile (simt_rb.cuh, simt_warp.cuh) on it, until all tiles are handed out.  No item waits on
 // another, so the kernel has no spin-waits.  With use_graph the counter reset
 // and the launch are captured once per problem set and replayed.
 #include <string.h>
@@ -16,6 +16,7 @@
 
 #include "pgk_internal.cuh"
 #include "simt_rb.cuh"
+#include "simt_warp.cuh"
 
 namespace pgk {
 
@@ -58,6 +59,46 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::MINB)
     }
 }
 
+// The same on single-warp 64 x 64 tiles of simt_warp.cuh, eight to an SM.  Bound by the
+// FMA pipe and by what a tile wastes on ragged edges, where 64 x 64 loses less than
+// 128-wide tiles; the next item is taken, and its problem searched for by the whole warp
+// (32 prefix sums at a time), before the current tile runs.
+__global__ void __launch_bounds__(32, 8)
+    k_grouped_wt(const GProb* __restrict__ probs, const int* __restrict__ prefix, int G, int total,
+                 int* counter) {
+    typedef Wt64<1> Cfg;
+    extern __shared__ float4 smem_gw4[];
+    const int lane = threadIdx.x;
+    auto take = [&] {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(counter, 1);
+        return i;   // valid in lane 0
+    };
+    int next = take();
+    for (;;) {
+        const int item = __shfl_sync(0xffffffffu, next, 0);
+        if (item >= total) break;
+        next = take();
+        int lo = 0, hi = G;   // the problem lies in [lo, hi): the largest g with prefix[g] <= item
+        while (hi - lo > 1) {
+            const int step = (hi - lo + 31) / 32, g = lo + lane * step;
+            const bool le = g < hi && __ldg(prefix + g) <= item;
+            lo += (__popc(__ballot_sync(0xffffffffu, le)) - 1) * step;
+            hi = min(hi, lo + step);
+        }
+        const GProb p = probs[lo];
+        int bm, bn;
+        grouped_tile_coords(item - __ldg(prefix + lo), p.tiles_m, p.tiles_n, bm, bn);
+        float* smem = reinterpret_cast<float*>(smem_gw4);
+        if (wt_vec(p.vecA, p.vecB, p.N, p.K))
+            WarpTile<Cfg, true>::run(p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, 0, p.K, bm * Cfg::BM,
+                                     bn * Cfg::BN, p.beta, p.vecC, lane, 0, smem);
+        else
+            WarpTile<Cfg, false>::run(p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, 0, p.K, bm * Cfg::BM,
+                                      bn * Cfg::BN, p.beta, p.vecC, lane, 0, smem);
+    }
+}
+
 struct GroupedVariant {
     int B0, B1, sr, s, BK;
     int bm, bn, smem, threads;
@@ -69,6 +110,12 @@ template <class Cfg>
 static cudaError_t launch_grouped(const GProb* t, const int* prefix, int G, int total, int* counter,
                                   int grid, cudaStream_t st) {
     k_grouped<Cfg><<<grid, Cfg::NT, Cfg::SMEM, st>>>(t, prefix, G, total, counter);
+    return cudaGetLastError();
+}
+
+static cudaError_t launch_grouped_wt(const GProb* t, const int* prefix, int G, int total, int* counter,
+                                     int grid, cudaStream_t st) {
+    k_grouped_wt<<<grid, Wt64<1>::THREADS, Wt64<1>::SMEM, st>>>(t, prefix, G, total, counter);
     return cudaGetLastError();
 }
 
@@ -85,6 +132,8 @@ static const GroupedVariant* grouped_table(int* n) {
         gv<16, 16, 8, 8, 8>(),  gv<16, 16, 8, 8, 16>(), gv<16, 16, 4, 4, 8>(),
         gv<16, 16, 8, 4, 8>(),  gv<16, 16, 4, 8, 8>(),  gv<8, 16, 8, 8, 8>(),
         gv<16, 8, 8, 8, 8>(),   gv<8, 8, 8, 8, 8>(),
+        {4, 8, 16, 8, 8, Wt64<1>::BM, Wt64<1>::BN, Wt64<1>::SMEM, Wt64<1>::THREADS,
+         (const void*)k_grouped_wt, launch_grouped_wt},
     };
     *n = (int)(sizeof(t) / sizeof(t[0]));
     return t;
@@ -226,8 +275,6 @@ static pgk_status enqueue(const GroupedVariant& v, void* dtable, int G, int tota
     return PGK_OK;
 }
 
-pgk_params default_params(int M, int N, int K, pgk_dtype dtype);
-
 }  // namespace pgk
 
 using namespace pgk;
@@ -247,7 +294,7 @@ extern "C" pgk_status pgk_gemm_grouped(int G, const pgk_problem* problems, pgk_d
     if (prog) {
         p = *prog;
     } else if (pgk_tune_cache_get(-G, 0, 0, PGK_F32, &p) != PGK_OK) {
-        pgk_params d = {16, 16, 4, 4, 8};
+        pgk_params d = {4, 8, 8, 16, 8};
         p = d;
     }
     const GroupedVariant* v = find_grouped(&p);

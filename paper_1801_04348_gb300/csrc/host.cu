@@ -343,13 +343,8 @@ static pgk_status select_any(const pgk_machine* m, const int* regs_table, int M,
 // ----------------------------------------------------------------- SIMT run
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-pgk_status run_simt_case(const pgk_case& c, int M, int N, int K, const float* A, int lda,
-                         const float* B, int ldb, float* C, int ldc, int beta, cudaStream_t st) {
-    std::vector<Variant>& r = registry();
-    if (c.variant_id < 0 || c.variant_id >= (int)r.size() || !r[c.variant_id].launch) {
-        set_error("case does not name a SIMT variant");
-        return PGK_ERR_INVALID_ARG;
-    }
+static SimtArgs simt_args(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C,
+                          int ldc, int beta) {
     SimtArgs a;
     a.M = M;
     a.N = N;
@@ -361,12 +356,24 @@ pgk_status run_simt_case(const pgk_case& c, int M, int N, int K, const float* A,
     a.C = C;
     a.ldc = ldc;
     a.beta = beta ? 1 : 0;
-    a.B0 = c.params.B0;
-    a.B1 = c.params.B1;
-    a.BK = c.params.tile;
+    a.B0 = a.B1 = a.BK = 0;
     a.vecA = aligned16(A) && lda % 4 == 0;
     a.vecB = aligned16(B) && ldb % 4 == 0;
     a.vecC = aligned16(C) && ldc % 4 == 0;
+    return a;
+}
+
+pgk_status run_simt_case(const pgk_case& c, int M, int N, int K, const float* A, int lda,
+                         const float* B, int ldb, float* C, int ldc, int beta, cudaStream_t st) {
+    std::vector<Variant>& r = registry();
+    if (c.variant_id < 0 || c.variant_id >= (int)r.size() || !r[c.variant_id].launch) {
+        set_error("case does not name a SIMT variant");
+        return PGK_ERR_INVALID_ARG;
+    }
+    SimtArgs a = simt_args(M, N, K, A, lda, B, ldb, C, ldc, beta);
+    a.B0 = c.params.B0;
+    a.B1 = c.params.B1;
+    a.BK = c.params.tile;
     cudaError_t e = r[c.variant_id].launch(a, c.smem_bytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "SIMT GEMM launch");
     return PGK_OK;
@@ -388,9 +395,11 @@ static pgk_status check_gemm_args(int M, int N, int K, const void* A, int lda, c
     return PGK_OK;
 }
 
+// Parameters of a call that names none, for the forms that still take one program
+// (FP32 plans its tile by shape: simt_wide_launch).
 pgk_params default_params(int M, int N, int K, pgk_dtype dtype) {
     pgk_params p;
-    if (dtype == PGK_F32 || dtype == PGK_I32) {
+    if (dtype == PGK_I32) {
         if ((long long)M * N >= 2048LL * 2048) {
             p.B0 = 16; p.B1 = 16; p.s = 8; p.sr = 8; p.tile = 8;
         } else if ((long long)M * N >= 256LL * 256) {
@@ -442,6 +451,11 @@ pgk_status gemm_device(int M, int N, int K, pgk_dtype dtype, const float* A, int
             p = pgk_params{128, 64, dtype == PGK_SPLIT_BF16 ? 3 : 4, 0, 0};
         } else if (learned_select(M, N, K, dtype, A, lda, B, ldb, C, ldc, beta, stream, &p) !=
                    PGK_OK) {
+            if (dtype == PGK_F32) {
+                const cudaError_t e =
+                    simt_wide_launch(simt_args(M, N, K, A, lda, B, ldb, C, ldc, beta), 0, stream);
+                return e == cudaSuccess ? PGK_OK : cuda_fail(e, "SIMT GEMM launch");
+            }
             p = default_params(M, N, K, dtype);
         }
     }

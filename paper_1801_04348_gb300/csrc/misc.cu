@@ -14,8 +14,6 @@
 
 namespace pgk {
 
-pgk_params default_params(int M, int N, int K, pgk_dtype dtype);
-
 // -------------------------------------------------------------- workspaces
 // One set of workspaces and one error word per device: a call on device d only
 // ever receives memory of device d (the current device of the calling thread).

@@ -47,6 +47,10 @@ struct Variant {
     int smem_fixed;             // dynamic shared memory of a fixed-shape variant
 };
 
+// FP32 product on the wide tiles of simt_warp.cuh, tile and K slices chosen for the shape
+// (tile = 0: any tile; else only that one).
+cudaError_t simt_wide_launch(const SimtArgs& p, int tile, cudaStream_t st);
+
 // Registration hooks, one per translation unit that defines variants.
 void register_simt_variants(std::vector<Variant>& v);
 void register_tc_variants(std::vector<Variant>& v);

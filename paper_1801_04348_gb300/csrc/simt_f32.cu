@@ -7,16 +7,22 @@
 //     run-time indexed register array would live in local memory).
 //     Leaves (4a,3a) and (3b,4a) of the case discussion.
 //   * "direct" family: no shared memory, one output per thread; leaf (3b,4b).
-//   * "rb" family: register-blocked sr x s micro tiles (simt_rb.cuh).  When the
-//     output has fewer tiles than SMs and K >= 4096 the launch splits K into
-//     slices (at least 1024 deep); slice partials land in a library workspace and
-//     a second kernel adds them in slice order.
+//   * "rb" family: register-blocked sr x s micro tiles (simt_rb.cuh, and simt_warp.cuh
+//     for sr = 16 and the 32 x 32 tile).  When the output has fewer tiles than SMs
+//     and K >= 4096 the launch splits K into slices (at least 1024 deep); slice
+//     partials land in a library workspace and a second kernel adds them in slice
+//     order.
+// Without parameters FP32 products run the wide tiles of simt_warp.cuh, tile and K
+// slices chosen by wt_plan.
 // Every variant handles arbitrary M, N, K >= 1 with predicated, zero-filled
 // tails (the paper's k loop drops the remainder of n / B0).
+#include <math.h>
+
 #include <algorithm>
 
 #include "pgk_internal.cuh"
 #include "simt_rb.cuh"
+#include "simt_warp.cuh"
 
 namespace pgk {
 
@@ -182,35 +188,45 @@ __global__ void k_splitk_reduce(SimtArgs p, const float* __restrict__ P, int spl
     }
 }
 
+// Fewer output tiles than the GPU holds resident blocks, on a long K: K is split into as
+// many slices as still fit in one wave of resident blocks (slices of at least 1024); a
+// wave and a few blocks would cost two waves.  Returns 1 where K is not split.
+static int split_k(const SimtArgs& p, long long tiles, const void* f, int threads, int smem,
+                   cudaError_t* err) {
+    *err = cudaSuccess;
+    pgk_machine m;
+    if (p.K < 4096 || current_machine(&m, NULL) != PGK_OK) return 1;
+    if (smem > 48 * 1024 &&
+        (*err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+        return 1;
+    int per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        per_sm = 1;
+    }
+    const long long slots = (long long)std::max(per_sm, 1) * m.sm_count;
+    if (tiles >= slots) return 1;
+    return std::min((int)std::min<long long>(slots / tiles, 16), p.K / 1024);
+}
+
+// The slices' partial products P (M x N each) added into C, in slice order.
+template <bool INT>
+static void launch_splitk_reduce(const SimtArgs& p, const float* P, int splits, cudaStream_t st) {
+    pgk_machine m;
+    const int sms = current_machine(&m, NULL) == PGK_OK ? m.sm_count : 1;
+    const long long total = (long long)p.M * p.N;
+    const int blocks = (int)std::min<long long>((total + 255) / 256, 4LL * sms);
+    k_splitk_reduce<INT><<<blocks, 256, 0, st>>>(p, P, splits);
+}
+
 template <class Cfg, bool INT>
 static cudaError_t launch_rb(const SimtArgs& p, int, cudaStream_t st) {
     const long long tiles =
         (long long)((p.M + Cfg::BM - 1) / Cfg::BM) * ((p.N + Cfg::BN - 1) / Cfg::BN);
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    // Fewer output tiles than the GPU holds resident blocks, on a long K: split K
-    // into as many slices as still fit in one wave of resident blocks (slices of at
-    // least 1024, a multiple of BK); a wave and a few blocks would cost two waves.
-    pgk_machine m;
-    int splits = 1;
-    if (p.K >= 4096 && current_machine(&m, NULL) == PGK_OK) {
-        if (Cfg::SMEM > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute((const void*)k_rb_splitk<Cfg, INT>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 Cfg::SMEM);
-            if (e != cudaSuccess) return e;
-        }
-        int per_sm = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_rb_splitk<Cfg, INT>,
-                                                          Cfg::NT, Cfg::SMEM) != cudaSuccess) {
-            cudaGetLastError();
-            per_sm = 1;
-        }
-        const long long slots = (long long)std::max(per_sm, 1) * m.sm_count;
-        if (tiles < slots) {
-            splits = (int)std::min<long long>(slots / tiles, 16);
-            splits = std::min(splits, p.K / 1024);
-        }
-    }
+    cudaError_t e;
+    int splits = split_k(p, tiles, (const void*)k_rb_splitk<Cfg, INT>, Cfg::NT, Cfg::SMEM, &e);
+    if (e != cudaSuccess) return e;
     if (splits >= 2) {
         const int kslice = ((p.K + splits - 1) / splits + Cfg::BK - 1) / Cfg::BK * Cfg::BK;
         splits = (p.K + kslice - 1) / kslice;
@@ -219,18 +235,129 @@ static cudaError_t launch_rb(const SimtArgs& p, int, cudaStream_t st) {
         if (!P) return cudaErrorMemoryAllocation;
         k_rb_splitk<Cfg, INT><<<dim3((unsigned)tiles, (unsigned)splits), Cfg::NT, Cfg::SMEM, st>>>(
             p, P, kslice);
-        const long long total = (long long)p.M * p.N;
-        const int blocks = (int)std::min<long long>((total + 255) / 256, 4LL * m.sm_count);
-        k_splitk_reduce<INT><<<blocks, 256, 0, st>>>(p, P, splits);
+        launch_splitk_reduce<INT>(p, P, splits, st);
         return cudaGetLastError();
     }
     if (Cfg::SMEM > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute((const void*)k_rb<Cfg, INT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+        e = cudaFuncSetAttribute((const void*)k_rb<Cfg, INT>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
         if (e != cudaSuccess) return e;
     }
     k_rb<Cfg, INT><<<(unsigned)tiles, Cfg::NT, Cfg::SMEM, st>>>(p);
     return cudaGetLastError();
+}
+
+// ------------------------------------------------------------- wide tiles
+typedef cudaError_t (*wt_launch_fn)(const SimtArgs&, int groups, float* P, cudaStream_t);
+
+// A wide-tile configuration and what a K step of one of its warps costs (SM cycles,
+// measured at K = 4096): alone on its scheduler, and each of several warps on it.
+struct WtKind {
+    int tile, warps, ks;
+    float alone, shared;
+    wt_launch_fn launch;
+};
+static const WtKind wt_kinds[] = {
+    {128, 4, 1, 179.f, 147.f, launch_wt<Wt128>},     {64, 1, 1, 179.f, 152.f, launch_wt<Wt64<1>>},
+    {64, 2, 2, 179.f, 152.f, launch_wt<Wt64<2>>},    {64, 4, 4, 179.f, 152.f, launch_wt<Wt64<4>>},
+    {64, 8, 8, 179.f, 152.f, launch_wt<Wt64<8>>},    {32, 1, 1, 58.f, 53.f, launch_wt<Wt32<1>>},
+    {32, 2, 2, 58.f, 53.f, launch_wt<Wt32<2>>},      {32, 4, 4, 58.f, 53.f, launch_wt<Wt32<4>>},
+    {32, 8, 8, 58.f, 53.f, launch_wt<Wt32<8>>},
+};
+
+struct WtPlan {
+    const WtKind* kind;
+    int groups;
+};
+
+// The wide tile, the K slices in a block and the groups of slices over blocks with the
+// smallest estimated time.  The busiest SM runs ceil(blocks / SMs) blocks, so that many
+// warps over its four schedulers; each takes its K steps at the measured cost; blocks that
+// do not fit at once start in rounds of 2000 cycles; partial tiles of a block meet in
+// shared memory, those of several groups in the workspace and a second launch (9000
+// cycles and the traffic).  Against a sweep of all plans over 22 shapes (32 to 4096 a
+// side, ragged and unaligned ones) the estimate's choice is within 10 % of the fastest;
+// 256^3 runs in 6.2 us (64 x 64 tiles of 256 threads: 14.4), 1024^3 in 47 (94 without
+// slices), 2048^3 in 283 (331 with 128 x 128 tiles, 256 of them on 304 places).
+// More than one group needs a workspace, shared per device, which short products never
+// used: it is limited to K >= 4096 with few tiles, where every program splits K, and left
+// out while the stream is being captured (a workspace cannot grow there).
+static WtPlan wt_plan(int M, int N, int K, int sms, bool groups_allowed, int tile) {
+    WtPlan best = {nullptr, 1};
+    double best_t = 0;
+    const long long t64 = (long long)((M + 63) / 64) * ((N + 63) / 64);
+    const int max_groups = groups_allowed && K >= 4096 && t64 <= sms ? 16 : 1;
+    for (const WtKind& k : wt_kinds) {
+        if (tile && k.tile != tile) continue;
+        const long long tiles = (long long)((M + k.tile - 1) / k.tile) * ((N + k.tile - 1) / k.tile);
+        for (int g = 1; g <= max_groups; g *= 2) {
+            if (k.ks * g > 1 && K / (k.ks * g) < 32) break;
+            const double steps = (double)(((long long)K + k.ks * g - 1) / (k.ks * g));
+            const double blocks = (double)((tiles * g + sms - 1) / sms);
+            const double per_sched = ceil(blocks * k.warps / 4);
+            const double resident = k.tile == 32 ? 4 : 2;   // warps per scheduler (registers)
+            double t = steps * (per_sched <= 1 ? k.alone : k.shared * per_sched) +
+                       2000 * ceil(per_sched / resident);
+            if (k.ks > 1) t += blocks * (k.ks * k.tile * k.tile / 16 + 300);
+            if (g > 1) t += 9000 + (double)g * M * N * 8 / 3400;
+            if (!best.kind || t < best_t) {
+                best = {&k, g};
+                best_t = t;
+            }
+        }
+    }
+    return best;
+}
+
+// Runs a plan; a failed workspace allocation falls back to one group of slices.
+static cudaError_t run_wt(const SimtArgs& p, const WtPlan& plan, cudaStream_t st) {
+    if (plan.groups > 1) {
+        pgk_status ws;
+        float* P = (float*)workspace(WS_SPLITK, sizeof(float) * (size_t)plan.groups * p.M * p.N, &ws);
+        if (P) {
+            const cudaError_t e = plan.kind->launch(p, plan.groups, P, st);
+            if (e != cudaSuccess) return e;
+            launch_splitk_reduce<false>(p, P, plan.groups, st);
+            return cudaGetLastError();
+        }
+    }
+    return plan.kind->launch(p, 1, nullptr, st);
+}
+
+// FP32 product without parameters (tile = 0), or with the 32 x 32 program's K slices.
+cudaError_t simt_wide_launch(const SimtArgs& p, int tile, cudaStream_t st) {
+    pgk_machine m;
+    if (current_machine(&m, NULL) != PGK_OK) return cudaErrorInvalidDevice;
+    WtPlan plan = wt_plan(p.M, p.N, p.K, m.sm_count, true, tile);
+    if (plan.groups > 1) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            plan = wt_plan(p.M, p.N, p.K, m.sm_count, false, tile);
+        }
+    }
+    return run_wt(p, plan, st);
+}
+
+// The wide-tile programs: one slice per block, K split over blocks as in launch_rb.
+template <class Cfg>
+static cudaError_t launch_wt_program(const SimtArgs& p, int, cudaStream_t st) {
+    const long long tiles =
+        (long long)((p.M + Cfg::BM - 1) / Cfg::BM) * ((p.N + Cfg::BN - 1) / Cfg::BN);
+    cudaError_t e;
+    const int splits = split_k(p, tiles, (const void*)k_wt<Cfg, false>, Cfg::THREADS, Cfg::SMEM, &e);
+    if (e != cudaSuccess) return e;
+    if (splits < 2) return launch_wt<Cfg>(p, 1, nullptr, st);
+    pgk_status ws;
+    float* P = (float*)workspace(WS_SPLITK, sizeof(float) * (size_t)splits * p.M * p.N, &ws);
+    if (!P) return cudaErrorMemoryAllocation;
+    if ((e = launch_wt<Cfg>(p, splits, P, st)) != cudaSuccess) return e;
+    launch_splitk_reduce<false>(p, P, splits, st);
+    return cudaGetLastError();
+}
+
+static cudaError_t launch_wt32_program(const SimtArgs& p, int, cudaStream_t st) {
+    return simt_wide_launch(p, 32, st);
 }
 
 // ------------------------------------------------------------ registration
@@ -307,6 +434,13 @@ void register_simt_variants(std::vector<Variant>& v) {
     add_rb<16, 16, 16, 8, 8>(v);
     add_rb<16, 16, 16, 8, 16>(v);
     add_rb<16, 16, 8, 16, 16>(v);
+    // wide tiles: 128 x 128 of four warps, 64 x 64 of one warp, 32 x 32 with K slices
+    v.push_back(make_variant(PGK_FAM_RB, 8, 16, 8, 16, 8, 0, (const void*)k_wt<Wt128, false>,
+                             launch_wt_program<Wt128>, Wt128::SMEM));
+    v.push_back(make_variant(PGK_FAM_RB, 8, 16, 4, 8, 8, 0, (const void*)k_wt<Wt64<1>, false>,
+                             launch_wt_program<Wt64<1>>, Wt64<1>::SMEM));
+    v.push_back(make_variant(PGK_FAM_RB, 4, 8, 4, 8, 16, 0, (const void*)k_wt<Wt32<1>, false>,
+                             launch_wt32_program, Wt32<1>::SMEM));
 }
 
 }  // namespace pgk

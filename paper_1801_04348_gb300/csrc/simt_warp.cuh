@@ -1,0 +1,311 @@
+// FP32 SIMT tiles with wide micro tiles (programs with sr = 16 and the 32 x 32 tile).
+//
+// A thread holds TM x TN outputs in rows of four strided by 4 LM and columns of four
+// strided by 4 LN (the paper's coalesced stride, in float4 groups), as row pairs for the
+// paired FMA: the A fragment of a k comes out of shared memory already paired, and each
+// of the TN values of B is duplicated once and meets TM / 2 pairs.
+//
+// What bounds it: the FMA pipe.  With 16 x 8 outputs a k costs 6 shared-memory loads and
+// 16 register moves beside 64 paired FMAs (128 pipe cycles of a warp); the 8 x 8 micro
+// tile of simt_rb.cuh pays 4 loads and 16 moves for 32, keeps the pipe 76 % busy at
+// 4096^3 and runs at 55.9 TFLOP/s there (58.9 at 8192^3).  Measured on GB300 at 4096^3 and
+// 8192^3 (derived SIMT peak 80.5): 128 x 128 tiles of four warps 61.8 / 65.3, 64 x 64
+// tiles of a single warp 60.2 / 63.4; two resident blocks of the 128 x 128 tile, or eight
+// of the 64 x 64 one, fill the register file.  Deeper K tiles (16, 32) gain at most 1 %
+// or spill, fragment double buffering loses 4 %, and B stored duplicated in shared memory
+// (no moves) is bound by shared-memory bandwidth at 46.
+//
+// A single-warp tile needs no block barrier, and the warps of one block may take
+// consecutive slices of K (KS of them) and add their tiles in slice order through shared
+// memory: that fills the GPU where the output has few tiles, without a workspace or a
+// second launch.
+#pragma once
+
+#include <algorithm>
+#include <climits>
+
+#include "pgk_internal.cuh"
+#include "simt_rb.cuh"
+
+namespace pgk {
+
+// BM x BN tile by WGM x WGN warps of LM x LN lanes, TM x TN outputs per thread, K tiles of
+// BK, KS slices of K per block (KS > 1: WGM = WGN = 1, warp w takes slice w).
+template <int BM_, int BN_, int BK_, int WGM_, int WGN_, int LM_, int LN_, int TM_, int TN_, int KS_>
+struct WtCfg {
+    static constexpr int BM = BM_, BN = BN_, BK = BK_, WGM = WGM_, WGN = WGN_, LM = LM_, LN = LN_;
+    static constexpr int TM = TM_, TN = TN_, KS = KS_;
+    static constexpr int NW = WGM * WGN;           // warps that share one K slice
+    static constexpr int NT = 32 * NW;             // their threads
+    static constexpr int THREADS = NT * KS;
+    static constexpr int LDAS = BM + 4, LDBS = BN + 4;
+    static constexpr int A_ELEMS = BK * LDAS, B_ELEMS = BK * LDBS;
+    static constexpr int SLICE_FLOATS = 2 * (A_ELEMS + B_ELEMS);
+    static constexpr int STAGE_BYTES = 4 * SLICE_FLOATS * KS;
+    static constexpr int RED_BYTES = KS > 1 ? 4 * KS * BM * BN : 0;   // partial tiles, over the stages
+    static constexpr int SMEM = STAGE_BYTES > RED_BYTES ? STAGE_BYTES : RED_BYTES;
+    static constexpr int LA = BM * BK / 4 / NT, LB = BN * BK / 4 / NT;   // float4 per thread
+    // resident blocks: as many as 16 x 8 outputs (8 warps) or 8 x 4 outputs (16 warps) allow
+    static constexpr int MINB = (TM * TN >= 128 ? 8 : 16) / (NW * KS) > 0 ? (TM * TN >= 128 ? 8 : 16) / (NW * KS) : 1;
+    static_assert(WGM * LM * TM == BM && WGN * LN * TN == BN && LM * LN == 32, "tile = warps x lanes x outputs");
+    static_assert(LA * NT * 4 == BM * BK && LB * NT * 4 == BN * BK, "whole float4 per thread");
+    static_assert(KS == 1 || NW == 1, "K slices are single warps");
+    static_assert(TM % 4 == 0 && TN % 4 == 0 && BK % 4 == 0, "float4 groups");
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// VEC: A and B are read 16 bytes at a time, which needs their bases and row strides on
+// 16-byte boundaries and K and N multiples of 4 (a float4 then lies wholly inside or
+// outside the matrix).  Rows and columns beyond M and N are read at the last row or
+// column instead (their outputs are never stored), K beyond its end reads as zero.
+template <class Cfg, bool VEC>
+struct WarpTile {
+    static __device__ __forceinline__ void sync() {
+        if (Cfg::NW == 1) __syncwarp();
+        else __syncthreads();
+    }
+
+    // Output tile at (row0, col0) over k in [k_begin, k_end): acc and, for KS > 1, the sum
+    // over the block's slices, then C (+)= it.  tid: thread within its slice's warps; sl:
+    // the slice.  k_begin is a multiple of 4.
+    static __device__ __forceinline__ void run(const float* __restrict__ A, int lda,
+                                               const float* __restrict__ B, int ldb, float* C, int ldc,
+                                               int M, int N, int k_begin, int k_end, int row0, int col0,
+                                               int beta, int vecC, int tid, int sl, float* smem) {
+        constexpr int BK = Cfg::BK;
+        const int w = tid >> 5, l = tid & 31;
+        const int ta = l / Cfg::LN, tb = l % Cfg::LN;
+        const int ra0 = (w / Cfg::WGN) * (Cfg::LM * Cfg::TM) + 4 * ta;
+        const int cb0 = (w % Cfg::WGN) * (Cfg::LN * Cfg::TN) + 4 * tb;
+        float* As = smem + sl * Cfg::SLICE_FLOATS;
+        float* Bs = As + 2 * Cfg::A_ELEMS;
+        float4 ra[Cfg::LA];
+        // the thread's first float4 of A (row am, k 4 akq) and of B (k bk, columns 4 bnq)
+        const int am = tid / (BK / 4), akq = tid % (BK / 4);
+        const int bk = tid / (Cfg::BN / 4), bnq = tid % (Cfg::BN / 4);
+        constexpr int AM_STEP = Cfg::NT / (BK / 4), BK_STEP = Cfg::NT / (Cfg::BN / 4);
+        static_assert(Cfg::NT % (BK / 4) == 0 && Cfg::NT % (Cfg::BN / 4) == 0, "fixed column per thread");
+
+        auto load_a = [&](int k0) {
+            const int gk = k0 + 4 * akq;
+#pragma unroll
+            for (int i = 0; i < Cfg::LA; ++i) {
+                const int gm = min(row0 + am + i * AM_STEP, M - 1);
+                const float* p = A + (size_t)gm * lda + gk;
+                if (VEC) {
+                    ra[i] = gk < k_end ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                } else {
+                    ra[i].x = gk + 0 < k_end ? __ldg(p + 0) : 0.f;
+                    ra[i].y = gk + 1 < k_end ? __ldg(p + 1) : 0.f;
+                    ra[i].z = gk + 2 < k_end ? __ldg(p + 2) : 0.f;
+                    ra[i].w = gk + 3 < k_end ? __ldg(p + 3) : 0.f;
+                }
+            }
+        };
+        auto store_a = [&](int buf) {
+            float* d0 = As + buf * Cfg::A_ELEMS + 4 * akq * Cfg::LDAS + am;
+#pragma unroll
+            for (int i = 0; i < Cfg::LA; ++i) {
+                float* d = d0 + i * AM_STEP;
+                d[0] = ra[i].x;
+                d[Cfg::LDAS] = ra[i].y;
+                d[2 * Cfg::LDAS] = ra[i].z;
+                d[3 * Cfg::LDAS] = ra[i].w;
+            }
+        };
+        auto load_b = [&](int k0, int buf) {
+            const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(Bs + buf * Cfg::B_ELEMS + bk * Cfg::LDBS + 4 * bnq);
+            const int gn = col0 + 4 * bnq;
+#pragma unroll
+            for (int i = 0; i < Cfg::LB; ++i) {
+                const int gk = k0 + bk + i * BK_STEP;
+                const bool in = gk < k_end;
+                const float* p = B + (size_t)(in ? gk : 0) * ldb;   // (nothing is read when !in)
+                const uint32_t d = d0 + 4u * (uint32_t)(i * BK_STEP * Cfg::LDBS);
+                if (VEC) {
+                    cp_async16(d, p + min(gn, N - 4), in ? 16 : 0);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) cp_async4(d + 4u * u, p + min(gn + u, N - 1), in ? 4 : 0);
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+
+        uint64_t acc[Cfg::TM / 2][Cfg::TN];   // [i][j]: rows 2i and 2i + 1 of the thread, column j
+#pragma unroll
+        for (int i = 0; i < Cfg::TM / 2; ++i)
+#pragma unroll
+            for (int j = 0; j < Cfg::TN; ++j) acc[i][j] = 0ull;
+
+        load_a(k_begin);
+        load_b(k_begin, 0);
+        store_a(0);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        sync();
+        int cur = 0;
+        for (int k0 = k_begin; k0 < k_end;) {
+            const bool more = k_end - k0 > BK;
+            if (more) {
+                load_a(k0 + BK);
+                load_b(k0 + BK, cur ^ 1);
+            }
+            const float* as = As + cur * Cfg::A_ELEMS + ra0;
+            const float* bs = Bs + cur * Cfg::B_ELEMS + cb0;
+#pragma unroll
+            for (int k = 0; k < BK; ++k) {
+                uint64_t a2[Cfg::TM / 2];
+                float b[Cfg::TN];
+#pragma unroll
+                for (int i = 0; i < Cfg::TM / 4; ++i) {
+                    const float4 v = *reinterpret_cast<const float4*>(as + k * Cfg::LDAS + i * 4 * Cfg::LM);
+                    a2[2 * i] = pack2(v.x, v.y);
+                    a2[2 * i + 1] = pack2(v.z, v.w);
+                }
+#pragma unroll
+                for (int j = 0; j < Cfg::TN / 4; ++j) {
+                    const float4 v = *reinterpret_cast<const float4*>(bs + k * Cfg::LDBS + j * 4 * Cfg::LN);
+                    b[4 * j] = v.x;
+                    b[4 * j + 1] = v.y;
+                    b[4 * j + 2] = v.z;
+                    b[4 * j + 3] = v.w;
+                }
+#pragma unroll
+                for (int j = 0; j < Cfg::TN; ++j) {
+                    const uint64_t bj = pack2(b[j], b[j]);
+#pragma unroll
+                    for (int i = 0; i < Cfg::TM / 2; ++i) fma2(acc[i][j], a2[i], bj);
+                }
+            }
+            if (more) {
+                store_a(cur ^ 1);
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            sync();
+            cur ^= 1;
+            if (!more) break;
+            k0 += BK;
+        }
+
+        auto out4 = [&](int i, int j) {   // row i of the thread, columns 4 j .. 4 j + 3
+            return (i & 1) ? make_float4(hi32(acc[i / 2][4 * j]), hi32(acc[i / 2][4 * j + 1]),
+                                         hi32(acc[i / 2][4 * j + 2]), hi32(acc[i / 2][4 * j + 3]))
+                           : make_float4(lo32(acc[i / 2][4 * j]), lo32(acc[i / 2][4 * j + 1]),
+                                         lo32(acc[i / 2][4 * j + 2]), lo32(acc[i / 2][4 * j + 3]));
+        };
+        auto store4 = [&](float4 o, int gm, int gn) {
+            float* cp = C + (size_t)gm * ldc + gn;
+            if (vecC && gn + 3 < N) {
+                if (beta) {
+                    const float4 c = *reinterpret_cast<const float4*>(cp);
+                    o.x += c.x;
+                    o.y += c.y;
+                    o.z += c.z;
+                    o.w += c.w;
+                }
+                *reinterpret_cast<float4*>(cp) = o;
+            } else {
+                if (gn + 0 < N) cp[0] = beta ? cp[0] + o.x : o.x;
+                if (gn + 1 < N) cp[1] = beta ? cp[1] + o.y : o.y;
+                if (gn + 2 < N) cp[2] = beta ? cp[2] + o.z : o.z;
+                if (gn + 3 < N) cp[3] = beta ? cp[3] + o.w : o.w;
+            }
+        };
+        if (Cfg::KS == 1) {
+#pragma unroll
+            for (int i = 0; i < Cfg::TM; ++i) {
+                const int gm = row0 + ra0 + (i / 4) * 4 * Cfg::LM + i % 4;
+                if (gm < M) {
+#pragma unroll
+                    for (int j = 0; j < Cfg::TN / 4; ++j) store4(out4(i, j), gm, col0 + cb0 + j * 4 * Cfg::LN);
+                }
+            }
+            return;
+        }
+        // the slices' tiles meet in shared memory (over the stages, which no warp reads any
+        // more) and are added in slice order
+        __syncthreads();
+        float* part = smem + sl * (Cfg::BM * Cfg::BN);
+#pragma unroll
+        for (int i = 0; i < Cfg::TM; ++i) {
+            const int r = ra0 + (i / 4) * 4 * Cfg::LM + i % 4;
+#pragma unroll
+            for (int j = 0; j < Cfg::TN / 4; ++j)
+                *reinterpret_cast<float4*>(part + r * Cfg::BN + cb0 + j * 4 * Cfg::LN) = out4(i, j);
+        }
+        __syncthreads();
+        for (int e = sl * Cfg::NT + tid; e < Cfg::BM * Cfg::BN / 4; e += Cfg::THREADS) {
+            const int r = e / (Cfg::BN / 4), c = e % (Cfg::BN / 4) * 4;
+            if (row0 + r >= M || col0 + c >= N) continue;
+            float4 s = *reinterpret_cast<const float4*>(smem + 4 * e);
+#pragma unroll
+            for (int y = 1; y < Cfg::KS; ++y) {
+                const float4 v = *reinterpret_cast<const float4*>(smem + y * (Cfg::BM * Cfg::BN) + 4 * e);
+                s.x += v.x;
+                s.y += v.y;
+                s.z += v.z;
+                s.w += v.w;
+            }
+            store4(s, row0 + r, col0 + c);
+        }
+    }
+};
+
+// blockIdx.x: output tile; blockIdx.y: one of gridDim.y groups of KS consecutive K slices of
+// kper each.  With more than one group the partial products go to P (M x N each, in group
+// order), for a second launch to add.
+template <class Cfg, bool VEC>
+__global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_wt(SimtArgs p, float* P, int kper) {
+    extern __shared__ float4 smem_wt4[];
+    const int tiles_m = (p.M + Cfg::BM - 1) / Cfg::BM;
+    const int tiles_n = (p.N + Cfg::BN - 1) / Cfg::BN;
+    int bm, bn;
+    grouped_tile_coords(blockIdx.x, tiles_m, tiles_n, bm, bn);
+    const int tid = Cfg::KS > 1 ? threadIdx.x & 31 : threadIdx.x, sl = Cfg::KS > 1 ? threadIdx.x >> 5 : 0;
+    const int kb = (int)min((long long)p.K, (long long)((int)blockIdx.y * Cfg::KS + sl) * kper);
+    const int ke = kb + min(kper, p.K - kb);
+    const bool split = gridDim.y > 1;
+    WarpTile<Cfg, VEC>::run(p.A, p.lda, p.B, p.ldb, split ? P + (size_t)blockIdx.y * p.M * p.N : p.C,
+                            split ? p.N : p.ldc, p.M, p.N, kb, ke, bm * Cfg::BM, bn * Cfg::BN,
+                            split ? 0 : p.beta, split ? (p.N & 3) == 0 : p.vecC, tid, sl,
+                            reinterpret_cast<float*>(smem_wt4));
+}
+
+// Whether both operands may be read 16 bytes at a time (see WarpTile).
+__host__ __device__ inline bool wt_vec(int vecA, int vecB, int N, int K) {
+    return vecA && vecB && N % 4 == 0 && K % 4 == 0;
+}
+
+// The product as gridDim.y = groups groups of KS slices (groups > 1: P holds the partials).
+template <class Cfg>
+static cudaError_t launch_wt(const SimtArgs& p, int groups, float* P, cudaStream_t st) {
+    const long long tiles =
+        (long long)((p.M + Cfg::BM - 1) / Cfg::BM) * ((p.N + Cfg::BN - 1) / Cfg::BN);
+    if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    const int slices = groups * Cfg::KS;
+    const long long kper = std::min<long long>(
+        INT_MAX, ((p.K + (long long)slices - 1) / slices + Cfg::BK - 1) / Cfg::BK * Cfg::BK);
+    const bool vec = wt_vec(p.vecA, p.vecB, p.N, p.K);
+    const void* f = vec ? (const void*)k_wt<Cfg, true> : (const void*)k_wt<Cfg, false>;
+    if (Cfg::SMEM > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+        if (e != cudaSuccess) return e;
+    }
+    const dim3 grid((unsigned)tiles, (unsigned)groups);
+    if (vec) k_wt<Cfg, true><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);
+    else k_wt<Cfg, false><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);
+    return cudaGetLastError();
+}
+
+// 128 x 128 tiles of four warps, 64 x 64 and 32 x 32 tiles of one warp per K slice.
+typedef WtCfg<128, 128, 8, 1, 4, 8, 4, 16, 8, 1> Wt128;
+template <int KS> using Wt64 = WtCfg<64, 64, 8, 1, 1, 4, 8, 16, 8, KS>;
+template <int KS> using Wt32 = WtCfg<32, 32, 16, 1, 1, 4, 8, 8, 4, KS>;
+
+}  // namespace pgk

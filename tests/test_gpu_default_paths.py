@@ -5,7 +5,8 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1801_04348_gb300 import pgk
+from helpers import assert_fp32_gemm
+from paper_1801_04348_gb300 import inputs, pgk
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +32,63 @@ def test_transpose_without_parameters(dev, rows, cols, pad_s, pad_d, shift):
     pgk.transpose(src, dst[:, :rows])
     assert torch.equal(dst[:, :rows], src.t())
     assert (dst[:, rows:] == -7).all() and (d[:shift] == -7).all()
+
+
+# one tile and less of each wide tile, one more row, column or K step than a tile, K slices
+# in a block (few tiles), groups of them (K >= 4096) and 128 x 128 tiles (many)
+F32_SHAPES = [(1, 1, 1), (31, 33, 15), (32, 32, 64), (33, 31, 257), (64, 65, 255), (129, 127, 1000), (1, 700, 90),
+              (64, 64, 8192), (100, 36, 4100), (700, 660, 72), (2500, 2060, 20)]
+
+
+@pytest.mark.parametrize("M,N,K", F32_SHAPES)
+@pytest.mark.parametrize("pad,beta", [(0, 0), (4, 1), (1, 1)])
+def test_f32_without_parameters(dev, M, N, K, pad, beta):
+    """FP32 products on the planned tile and K slices: the element-wise FP32 bound, with
+    row strides that allow 128-bit accesses (K and N multiples of 4 and pad 0 or 4) and
+    that do not; nothing beyond column N is written; a second call gives the same bits."""
+    A, B = inputs.gemm_operands(M, N, K, seed=M + 3 * N + 5 * K)
+    C0 = inputs.uniform((M, N), 9)
+    Aw, Bw = (torch.full((r, c + pad), float("nan"), device=dev) for r, c in ((M, K), (K, N)))
+    Aw[:, :K], Bw[:, :N] = torch.from_numpy(A), torch.from_numpy(B)
+    got = []
+    for _ in range(2):
+        C = torch.full((M, N + pad), float("nan"), device=dev)
+        C[:, :N] = torch.from_numpy(C0)
+        pgk.gemm(Aw[:, :K], Bw[:, :N], C, pgk.F32, beta=beta, M=M, N=N, K=K)
+        got.append(C)
+    assert torch.equal(got[0][:, :N], got[1][:, :N]) and torch.isnan(got[0][:, N:]).all()
+    assert_fp32_gemm(got[0][:, :N].cpu().numpy(), A, B, C0=C0, beta=beta)
+
+
+def test_f32_without_parameters_in_a_graph(dev):
+    """A shape whose K is split over blocks through a workspace outside a capture runs
+    without one inside it, also where the workspace could not grow any more."""
+    M, N, K = 64, 64, 8192
+    A, B = inputs.gemm_operands(M, N, K, seed=1)
+    At, Bt, C = torch.from_numpy(A).to(dev), torch.from_numpy(B).to(dev), torch.zeros(M, N, device=dev)
+    pgk.shutdown()
+    pgk.gemm(At[:32, :32].contiguous(), Bt[:32].contiguous(), C[:32], pgk.F32)   # load the kernels' module
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        pgk.gemm(At, Bt, C, pgk.F32)
+    C.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert_fp32_gemm(C.cpu().numpy(), A, B)
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+def test_grouped_wide_tile_on_ragged_problems(dev, shift):
+    """The default grouped tile over problems around its 64 x 64 edges, some with bases
+    off 16-byte boundaries: every one equals the same tile program launched alone."""
+    dims = [(1, 1, 1), (64, 64, 8), (65, 63, 9), (128, 4, 100), (3, 130, 33), (200, 200, 1), (66, 68, 64)] * 7
+    trip = []
+    for i, (M, N, K) in enumerate(dims):
+        a, b = (torch.randn(n + shift, device=dev)[shift:] for n in (M * K, K * N))
+        trip.append((a.view(M, K), b.view(K, N), torch.full((M, N), float("nan"), device=dev)))
+    pgk.gemm_grouped(pgk.make_problems(trip), pgk.F32, pgk.params(4, 8, 8, 16, 8))
+    for A, B, C in trip:
+        one = torch.empty_like(C)
+        pgk.gemm(A, B, one, pgk.F32, pgk.params(4, 8, 8, 16, 8))
+        assert torch.equal(one, C)
+        assert_fp32_gemm(C.cpu().numpy(), A.cpu().numpy(), B.cpu().numpy())
