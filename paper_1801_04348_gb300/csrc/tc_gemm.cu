@@ -99,8 +99,8 @@ struct TcCfg {
     // chunk accumulators so the MMA can run three chunks ahead of the epilogue
     static constexpr int ACC_BUFS = (MODE == MODE_FP8 && BN == 128) ? 4 : 2;
     static constexpr int TMEM_COLS = ACC_BUFS * BN;
-    // epilogue staging: one 32 x 33 FP32 block per epilogue warp after the stage ring
-    static constexpr int XPOSE_BYTES = EPI_WARPS * 32 * 33 * 4;
+    // epilogue staging: one 32 x 32 FP32 block per epilogue warp after the stage ring
+    static constexpr int XPOSE_BYTES = EPI_WARPS * 32 * 32 * 4;
     static constexpr int SMEM_RAW = STAGES * STAGE_BYTES + FSTAGES * F_BYTES + XPOSE_BYTES + 1024;
     // at least 116 KB so that one CTA owns the SM (and its tensor memory)
     static constexpr int SMEM = SMEM_RAW > 118784 ? SMEM_RAW : 118784;
@@ -930,25 +930,80 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
         // -------------------------------------------------------- epilogue
         const int e = warp - 2;
         const int q = warp & 3;                       // TMEM lane quarter of this warp
-        // a thread holds 32 consecutive columns of its own row after tcgen05.ld; the
-        // block goes through this warp's shared staging (pitch 33: conflict-free both
-        // ways) so that every store instruction covers 32 consecutive columns of a row
-        float* xp = reinterpret_cast<float*>(tiles + (size_t)Cfg::STAGES * Cfg::STAGE_BYTES +
-                                             (size_t)Cfg::FSTAGES * Cfg::F_BYTES) +
-                    e * (32 * 33);
+        // A thread holds 32 consecutive columns of its own row after tcgen05.ld; the block
+        // goes through this warp's staging (32 rows of 128 bytes, 16-byte chunk j of row r at
+        // j ^ (r mod 8): conflict-free both ways) so that C is accessed along its rows.
+        // Where C's rows allow it an access covers four rows of 128 bytes, 16 bytes per lane
+        // (8 stores for the block); otherwise one row of 32 columns (32 stores).  With beta = 1
+        // 16 rows of C are read before the first of them is written: the wait for memory, taken
+        // row by row, was most of a small product's time (513 x 1030 x 777, unaligned rows, the
+        // launch alone: split 29.6 -> 16.3 us, BF16 42.9 -> 15.2).  With beta = 0 the wide
+        // stores give 8192 x 1024 x 4096 in BF16 57.0 -> 53.5 us.
+        float4* xp = reinterpret_cast<float4*>(tiles + (size_t)Cfg::STAGES * Cfg::STAGE_BYTES +
+                                               (size_t)Cfg::FSTAGES * Cfg::F_BYTES) +
+                     e * (32 * 8);
         auto store_block = [&](const float (&v)[32], int row0, int cb, int M, int N, float* C,
                                int ldc, int beta) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) xp[lane * 33 + j] = v[j];
+            for (int j = 0; j < 8; ++j)
+                xp[lane * 8 + (j ^ (lane & 7))] =
+                    make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             __syncwarp();
-            const int col = cb + lane;
-#pragma unroll 4
-            for (int rr = 0; rr < 32; ++rr) {
-                const int row = row0 + rr;
-                if (row < M && col < N) {
-                    float* cp = C + (size_t)row * ldc + col;
-                    const float x = xp[rr * 33 + lane];
-                    *cp = beta ? *cp + x : x;
+            // (opaque here, so that no row address outlives a block: the chunked forms hold
+            // up to 128 sums in registers meanwhile)
+            asm volatile("" : "+r"(ldc), "+r"(row0));
+            if (((uintptr_t)C & 15u) == 0 && (ldc & 3) == 0 && cb + 32 <= N) {
+                const int rq = lane >> 3, ch = lane & 7;   // row within four, chunk
+                const int left = M - row0 - rq;            // rows 4 i below it exist
+                float* cp = C + (size_t)(row0 + rq) * ldc + cb + 4 * ch;
+                const size_t step = (size_t)ldc * 4;
+                if (beta) {
+#pragma unroll 1
+                    for (int h = 0; h < 8; h += 4) {
+                        float4 c[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            c[i] = 4 * (h + i) < left ? *reinterpret_cast<const float4*>(cp + i * step)
+                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int r = 4 * (h + i) + rq;
+                            const float4 x = xp[r * 8 + (ch ^ (r & 7))];
+                            if (4 * (h + i) < left)
+                                *reinterpret_cast<float4*>(cp + i * step) =
+                                    make_float4(c[i].x + x.x, c[i].y + x.y, c[i].z + x.z, c[i].w + x.w);
+                        }
+                        cp += 4 * step;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = 4 * i + rq;
+                        if (4 * i < left) *reinterpret_cast<float4*>(cp) = xp[r * 8 + (ch ^ (r & 7))];
+                        cp += step;
+                    }
+                }
+            } else if (cb + lane < N) {
+                const float* xs = reinterpret_cast<const float*>(xp) + (lane & 3);
+                float* cp = C + (size_t)row0 * ldc + cb + lane;
+                const int q4 = lane >> 2, rows = min(32, M - row0);
+                if (beta) {
+#pragma unroll 1
+                    for (int h = 0; h < 32; h += 16) {
+                        float c[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) c[i] = h + i < rows ? cp[(size_t)i * ldc] : 0.f;
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (h + i < rows) cp[(size_t)i * ldc] = c[i] + xs[(h + i) * 32 + ((q4 ^ (i & 7)) << 2)];
+                        cp += (size_t)16 * ldc;
+                    }
+                } else {
+#pragma unroll 8
+                    for (int r = 0; r < rows; ++r) {
+                        *cp = xs[r * 32 + ((q4 ^ (r & 7)) << 2)];
+                        cp += ldc;
+                    }
                 }
             }
             __syncwarp();
