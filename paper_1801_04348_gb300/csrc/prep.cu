@@ -6,6 +6,7 @@
 // tensor-core kernels read.  All are HBM-bound streaming kernels.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
+#include <string.h>
 
 #include <algorithm>
 #include <climits>
@@ -14,121 +15,159 @@
 
 namespace pgk {
 
-__device__ __forceinline__ uint16_t bf16_bits(float x) {
-    return __bfloat16_as_ushort(__float2bfloat16_rn(x));
-}
-
-__device__ __forceinline__ float bf16_value(uint16_t b) {
-    return __bfloat162float(__ushort_as_bfloat16(b));
-}
-
-// MODE 0: dst0 = bf16(x).  MODE 1: dst0 = hi, dst1 = lo.
+// MODE 0: h = bf16(x) of two values, the first in the lower half.  MODE 1: also
+// l = bf16(x - h), with x - h exact in FP32.
 template <int MODE>
-__device__ __forceinline__ void convert_one(float x, uint16_t& h, uint16_t& l) {
-    h = bf16_bits(x);
-    if (MODE == 1) l = bf16_bits(x - bf16_value(h));
-}
-
-// Row-major conversion: each thread handles 4 consecutive columns.
-template <int MODE>
-__global__ void k_cvt_rows(int rows, int cols, const float* __restrict__ src, int lds,
-                           uint16_t* __restrict__ d0, uint16_t* __restrict__ d1, int ldd, int vec) {
-    const int cq = (cols + 3) / 4;
-    const long long total = (long long)rows * cq;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(i / cq);
-        const int c = (int)(i - (long long)r * cq) * 4;
-        const float* s = src + (size_t)r * lds + c;
-        float v[4];
-        if (vec && c + 3 < cols) {
-            const float4 f = __ldg(reinterpret_cast<const float4*>(s));
-            v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = (c + u < cols) ? __ldg(s + u) : 0.f;
-        }
-        uint16_t h[4], l[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) convert_one<MODE>(v[u], h[u], l[u]);
-        uint16_t* o0 = d0 + (size_t)r * ldd + c;
-        uint16_t* o1 = MODE == 1 ? d1 + (size_t)r * ldd + c : nullptr;
-        if (vec && c + 3 < cols) {
-            *reinterpret_cast<uint2*>(o0) =
-                make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
-            if (MODE == 1)
-                *reinterpret_cast<uint2*>(o1) =
-                    make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c + u < cols) {
-                    o0[u] = h[u];
-                    if (MODE == 1) o1[u] = l[u];
-                }
-        }
+__device__ __forceinline__ void convert_two(float x, float y, uint32_t& h, uint32_t& l) {
+    const __nv_bfloat162 hp = __floats2bfloat162_rn(x, y);
+    h = *reinterpret_cast<const uint32_t*>(&hp);
+    if (MODE == 1) {
+        const float2 f = __bfloat1622float2(hp);
+        const __nv_bfloat162 lp = __floats2bfloat162_rn(x - f.x, y - f.y);
+        l = *reinterpret_cast<const uint32_t*>(&lp);
     }
 }
 
-// Transposed conversion through a 64 x 64 shared tile: src rows are read as
-// float4 (coalesced along src rows), each dst row (a src column) is written as
-// 32-bit pairs of BF16 values (a full 128-byte segment per warp).
+// Eight consecutive destination entries (n of them inside), one 128-bit store per plane
+// where the destination allows it.
 template <int MODE>
-__global__ void __launch_bounds__(256) k_cvt_transpose(int rows, int cols,
-                                                       const float* __restrict__ src, int lds,
-                                                       uint16_t* __restrict__ d0,
-                                                       uint16_t* __restrict__ d1, int ldd,
-                                                       int vec_in, int pair_out) {
-    __shared__ float t[64][65];
-    const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+__device__ __forceinline__ void store_eight(const float (&v)[8], uint16_t* __restrict__ o0,
+                                            uint16_t* __restrict__ o1, int n, int vec) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) convert_two<MODE>(v[2 * u], v[2 * u + 1], h[u], l[u]);
+    if (vec && n >= 8) {
+        *reinterpret_cast<uint4*>(o0) = make_uint4(h[0], h[1], h[2], h[3]);
+        if (MODE == 1) *reinterpret_cast<uint4*>(o1) = make_uint4(l[0], l[1], l[2], l[3]);
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (u < n) {
+            o0[u] = (uint16_t)(h[u / 2] >> (16 * (u & 1)));
+            if (MODE == 1) o1[u] = (uint16_t)(l[u / 2] >> (16 * (u & 1)));
+        }
+}
+
+// Four of them, one 64-bit store per plane.
+template <int MODE>
+__device__ __forceinline__ void store_four(float4 v, uint16_t* __restrict__ o0, uint16_t* __restrict__ o1,
+                                           int n, int vec) {
+    uint32_t h[2], l[2];
+    convert_two<MODE>(v.x, v.y, h[0], l[0]);
+    convert_two<MODE>(v.z, v.w, h[1], l[1]);
+    if (vec && n >= 4) {
+        *reinterpret_cast<uint2*>(o0) = make_uint2(h[0], h[1]);
+        if (MODE == 1) *reinterpret_cast<uint2*>(o1) = make_uint2(l[0], l[1]);
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (u < n) {
+            o0[u] = (uint16_t)(h[u / 2] >> (16 * (u & 1)));
+            if (MODE == 1) o1[u] = (uint16_t)(l[u / 2] >> (16 * (u & 1)));
+        }
+}
+
+// One 64 x 64 item at (r0, c0) of a source of rows x cols (zero outside), by a block of
+// 256 threads.  !TRANS: destination row r holds source row r, columns up to `width`.
+// TRANS: destination row c holds source column c, entries (source rows) up to `width`.
+// vec_in: source rows allow 128-bit loads; vec_out: destination rows 128-bit stores.
+// Bound by HBM: a thread has 64 bytes of loads in flight before its first store, segments
+// are 256 bytes of a source row and 128 of a destination row.  t is the block's shared
+// tile (a pitch of 65 words: the transposed reads of a warp meet at most two to a bank);
+// the block synchronises before it may be used again.
+template <int MODE, bool TRANS>
+__device__ __forceinline__ void cvt_item(const float* __restrict__ src, int lds, int rows, int cols,
+                                         int width, int vec_in, int vec_out, int r0, int c0,
+                                         uint16_t* __restrict__ d0, uint16_t* __restrict__ d1,
+                                         long long ldd, float (*t)[65]) {
     const int tid = threadIdx.x;
+    if (vec_in) {
+        float4 f[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int idx = tid + i * 256;
-        const int r = idx >> 4, c = (idx & 15) * 4;
-        const int gr = r0 + r, gc = c0 + c;
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (gr < rows) {
-            const float* sp = src + (size_t)gr * lds + gc;
-            if (vec_in && gc + 3 < cols) {
-                const float4 f = __ldg(reinterpret_cast<const float4*>(sp));
-                v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + tid / 16 + i * 16, c = c0 + tid % 16 * 4;
+            const int n = r < rows ? cols - c : 0;
+            const float* p = src + (size_t)r * lds + c;
+            f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (n >= 4) {
+                f[i] = __ldg(reinterpret_cast<const float4*>(p));
             } else {
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (gc + u < cols) v[u] = __ldg(sp + u);
+                if (n > 0) f[i].x = __ldg(p);
+                if (n > 1) f[i].y = __ldg(p + 1);
+                if (n > 2) f[i].z = __ldg(p + 2);
             }
         }
+        if (!TRANS) {
+            // kept rows: 16 lanes cover a row both ways (8-byte stores, 128 bytes a row)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) t[r][c + u] = v[u];
+            for (int i = 0; i < 4; ++i) {
+                const int r = r0 + tid / 16 + i * 16, c = c0 + tid % 16 * 4;
+                const size_t o = (size_t)((long long)r * ldd + c);
+                if (r < rows) store_four<MODE>(f[i], d0 + o, MODE == 1 ? d1 + o : nullptr, width - c, vec_out);
+            }
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float* o = &t[tid / 16 + i * 16][tid % 16 * 4];
+            o[0] = f[i].x;
+            o[1] = f[i].y;
+            o[2] = f[i].z;
+            o[3] = f[i].w;
+        }
+    } else {
+        float f[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int r = r0 + tid / 64 + i * 4, c = c0 + tid % 64;
+            f[i] = r < rows && c < cols ? __ldg(src + (size_t)r * lds + c) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) t[tid / 64 + i * 4][tid % 64] = f[i];
     }
     __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int c = warp * 8 + j;           // dst row c0 + c
-        const int gc = c0 + c;
-        if (gc >= cols) break;
-        const int gr = r0 + 2 * lane;         // dst columns gr, gr + 1
-        uint16_t h0, l0, h1, l1;
-        convert_one<MODE>(t[2 * lane][c], h0, l0);
-        convert_one<MODE>(t[2 * lane + 1][c], h1, l1);
-        uint16_t* o0 = d0 + (size_t)gc * ldd + gr;
-        uint16_t* o1 = MODE == 1 ? d1 + (size_t)gc * ldd + gr : nullptr;
-        if (pair_out && gr + 1 < rows) {
-            *reinterpret_cast<uint32_t*>(o0) = h0 | ((uint32_t)h1 << 16);
-            if (MODE == 1) *reinterpret_cast<uint32_t*>(o1) = l0 | ((uint32_t)l1 << 16);
-        } else {
-            if (gr < rows) {
-                o0[0] = h0;
-                if (MODE == 1) o1[0] = l0;
-            }
-            if (gr + 1 < rows) {
-                o0[1] = h1;
-                if (MODE == 1) o1[1] = l1;
-            }
-        }
+    for (int i = 0; i < 2; ++i) {
+        const int a = tid / 8 + i * 32, b = tid % 8 * 8;   // destination row and first entry in the item
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = TRANS ? t[b + u][a] : t[a][b + u];
+        const int gr = (TRANS ? c0 : r0) + a, ge = (TRANS ? r0 : c0) + b;
+        const size_t o = (size_t)((long long)gr * ldd + ge);
+        if (gr < (TRANS ? cols : rows))
+            store_eight<MODE>(v, d0 + o, MODE == 1 ? d1 + o : nullptr, width - ge, vec_out);
     }
+    __syncthreads();
+}
+
+// One operand of a conversion launch: `items` 64 x 64 items over its source (zero: none).
+struct CvtOp {
+    const float* src;
+    uint16_t *d0, *d1;
+    int lds, ldd, rows, cols, width;
+    int vec_in, vec_out;
+    int items, item_cols;   // items, and items along a row of the source
+};
+
+// Operand a (rows kept) takes the first a.items blocks, operand b (transposed) the rest:
+// both operands of a product in one launch.  Measured on GB300 at 8192^2 (before: one
+// thread per four columns with a 64-bit division, and 4-byte transposed stores): split
+// 86 -> 80 us kept, 92 -> 82 transposed (6.6 TB/s, a copy's rate), BF16 68 -> 61 and 72 ->
+// 61; 8191 x 8193 without 128-bit accesses 201 -> 82 and 96 -> 87.  Kept rows written 16
+// bytes a lane load every other half sector and lost 7 %.
+template <int MODE>
+__global__ void __launch_bounds__(256) k_cvt(const CvtOp a, const CvtOp b) {
+    __shared__ float t[64][65];
+    const int i = blockIdx.x;
+    if (i < a.items)
+        cvt_item<MODE, false>(a.src, a.lds, a.rows, a.cols, a.width, a.vec_in, a.vec_out,
+                              i / a.item_cols * 64, i % a.item_cols * 64, a.d0, a.d1, a.ldd, t);
+    else
+        cvt_item<MODE, true>(b.src, b.lds, b.rows, b.cols, b.width, b.vec_in, b.vec_out,
+                             (i - a.items) / b.item_cols * 64, (i - a.items) % b.item_cols * 64, b.d0, b.d1,
+                             b.ldd, t);
 }
 
 // Four consecutive elements of row r starting at column c (c a multiple of 4),
@@ -300,28 +339,64 @@ static pgk_status check_prep(int rows, int cols, const void* src, int lds, const
     return PGK_OK;
 }
 
-template <int MODE>
-static pgk_status launch_cvt(int rows, int cols, const float* src, int lds, uint16_t* d0,
-                             uint16_t* d1, int ldd, int transpose, cudaStream_t st) {
-    if (transpose) {
-        dim3 grid((cols + 63) / 64, (rows + 63) / 64);
-        if (grid.y > 65535) {
-            set_error("too many rows for the transposing conversion");
-            return PGK_ERR_INVALID_ARG;
-        }
-        const int vec_in = aligned(src, 16) && lds % 4 == 0;
-        const int pair_out = aligned(d0, 4) && ldd % 2 == 0 && (MODE == 0 || aligned(d1, 4));
-        k_cvt_transpose<MODE><<<grid, 256, 0, st>>>(rows, cols, src, lds, d0, d1, ldd, vec_in,
-                                                    pair_out);
-    } else {
-        const int vec = aligned(src, 16) && lds % 4 == 0 && aligned(d0, 8) && ldd % 4 == 0 &&
-                        (MODE == 0 || aligned(d1, 8));
-        const long long work = (long long)rows * ((cols + 3) / 4);
-        const int blocks = (int)std::min<long long>((work + 255) / 256, 152LL * 16);
-        k_cvt_rows<MODE><<<blocks, 256, 0, st>>>(rows, cols, src, lds, d0, d1, ldd, vec);
+// Describes one operand; width: destination entries to write per row (>= the source's).
+static bool cvt_op(CvtOp* o, int mode, int rows, int cols, const float* src, int lds,
+                   uint16_t* d0, uint16_t* d1, int ldd, int width) {
+    const long long ir = ((long long)rows + 63) / 64, ic = ((long long)cols + 63) / 64;
+    if (ir * ic > INT_MAX / 2) return false;
+    o->src = src;
+    o->d0 = d0;
+    o->d1 = d1;
+    o->lds = lds;
+    o->ldd = ldd;
+    o->rows = rows;
+    o->cols = cols;
+    o->width = width;
+    o->vec_in = aligned(src, 16) && lds % 4 == 0;
+    o->vec_out = aligned(d0, 16) && ldd % 8 == 0 && (mode == 0 || aligned(d1, 16));
+    o->items = (int)(ir * ic);
+    o->item_cols = (int)ic;
+    return true;
+}
+
+static pgk_status launch_cvt_ops(int mode, const CvtOp& a, const CvtOp& b, cudaStream_t st) {
+    const unsigned grid = (unsigned)a.items + (unsigned)b.items;
+    if (b.rows > 65535 * 64) {
+        set_error("too many rows for the transposing conversion");
+        return PGK_ERR_INVALID_ARG;
     }
+    if (mode == 0) k_cvt<0><<<grid, 256, 0, st>>>(a, b);
+    else k_cvt<1><<<grid, 256, 0, st>>>(a, b);
     PGK_CUDA_TRY(cudaGetLastError(), "conversion launch");
     return PGK_OK;
+}
+
+static pgk_status launch_cvt(int mode, int rows, int cols, const float* src, int lds, uint16_t* d0,
+                             uint16_t* d1, int ldd, int transpose, cudaStream_t st) {
+    CvtOp op[2];
+    memset(op, 0, sizeof(op));
+    if (!cvt_op(&op[transpose ? 1 : 0], mode, rows, cols, src, lds, d0, d1, ldd,
+                transpose ? rows : cols)) {
+        set_error("matrix too large for one conversion launch");
+        return PGK_ERR_INVALID_ARG;
+    }
+    return launch_cvt_ops(mode, op[0], op[1], st);
+}
+
+// Both operands of a product, A (M x K) and, unless b0 is NULL, B (K x N) transposed, into
+// workspaces of row stride Kp (a multiple of 16): one launch.
+pgk_status launch_cvt_operands(int mode, int M, int N, int K, const float* A, int lda, uint16_t* a0,
+                               uint16_t* a1, const float* B, int ldb, uint16_t* b0, uint16_t* b1, int Kp,
+                               cudaStream_t st) {
+    CvtOp op[2];
+    memset(op, 0, sizeof(op));
+    if ((a0 && !cvt_op(&op[0], mode, M, K, A, lda, a0, a1, Kp, Kp)) ||
+        (b0 && !cvt_op(&op[1], mode, K, N, B, ldb, b0, b1, Kp, Kp))) {
+        set_error("operands too large for one conversion launch");
+        return PGK_ERR_INVALID_ARG;
+    }
+    if (op[0].items + op[1].items == 0) return PGK_OK;
+    return launch_cvt_ops(mode, op[0], op[1], st);
 }
 
 pgk_status launch_quant_fp8(int rows, int cols, const float* src, int lds, uint8_t* dst, int ldd,
@@ -357,76 +432,11 @@ template <int MODE, bool TRANS>
 __device__ __forceinline__ void cvt_grouped_item(const GCvt& q, int local, uint16_t* __restrict__ d0,
                                                  uint16_t* __restrict__ d1, long long ldd,
                                                  float (*t)[65]) {
-    const int tid = threadIdx.x;
-    // tile grid over the padded source: TRANS covers width x cols, else rows x width
-    const int tcols = TRANS ? (q.cols + 63) / 64 : (q.width + 63) / 64;
-    const int r0 = (local / tcols) * 64, c0 = (local % tcols) * 64;
-    if (!TRANS) {
-        // direct: 64 rows x 64 columns, 4 quads per thread, zeros beyond cols
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int idx = tid + i * 256;
-            const int r = r0 + (idx >> 4), c = c0 + (idx & 15) * 4;
-            if (r >= q.rows || c >= q.width) continue;
-            float v[4];
-            const float* sp = q.src + (size_t)r * q.lds + c;
-            if (q.vec && c + 3 < q.cols) {
-                const float4 f = __ldg(reinterpret_cast<const float4*>(sp));
-                v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-            } else {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = (c + u < q.cols) ? __ldg(sp + u) : 0.f;
-            }
-            uint16_t h[4], l[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) convert_one<MODE>(v[u], h[u], l[u]);
-            const size_t o = (size_t)(q.dst_row + r) * ldd + c;   // width is a multiple of 4
-            *reinterpret_cast<uint2*>(d0 + o) =
-                make_uint2(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16));
-            if (MODE == 1)
-                *reinterpret_cast<uint2*>(d1 + o) =
-                    make_uint2(l[0] | ((uint32_t)l[1] << 16), l[2] | ((uint32_t)l[3] << 16));
-        }
-    } else {
-        // transposed: source rows r0 .. r0 + 63 (zeros beyond rows), columns c0 .. c0 + 63
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int idx = tid + i * 256;
-            const int r = idx >> 4, c = (idx & 15) * 4;
-            const int gr = r0 + r, gc = c0 + c;
-            float v[4] = {0.f, 0.f, 0.f, 0.f};
-            if (gr < q.rows) {
-                const float* sp = q.src + (size_t)gr * q.lds + gc;
-                if (q.vec && gc + 3 < q.cols) {
-                    const float4 f = __ldg(reinterpret_cast<const float4*>(sp));
-                    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-                } else {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (gc + u < q.cols) v[u] = __ldg(sp + u);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) t[r][c + u] = v[u];
-        }
-        __syncthreads();
-        const int warp = tid >> 5, lane = tid & 31;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c = warp * 8 + j;            // destination row dst_row + c0 + c
-            const int gc = c0 + c;
-            const int gr = r0 + 2 * lane;          // destination columns gr, gr + 1
-            if (gc < q.cols && gr < q.width) {     // width is even
-                uint16_t h0, l0, h1, l1;
-                convert_one<MODE>(t[2 * lane][c], h0, l0);
-                convert_one<MODE>(t[2 * lane + 1][c], h1, l1);
-                const size_t o = (size_t)(q.dst_row + gc) * ldd + gr;
-                *reinterpret_cast<uint32_t*>(d0 + o) = h0 | ((uint32_t)h1 << 16);
-                if (MODE == 1) *reinterpret_cast<uint32_t*>(d1 + o) = l0 | ((uint32_t)l1 << 16);
-            }
-        }
-        __syncthreads();   // the tile is reused by the next item
-    }
+    // item grid over the padded source: TRANS covers width x cols, else rows x width
+    const int icols = TRANS ? (q.cols + 63) / 64 : (q.width + 63) / 64;
+    const size_t o = (size_t)q.dst_row * ldd;
+    cvt_item<MODE, TRANS>(q.src, q.lds, q.rows, q.cols, q.width, q.vec, 1, local / icols * 64,
+                          local % icols * 64, d0 + o, MODE == 1 ? d1 + o : nullptr, ldd, t);
 }
 
 // Both operands of every problem in one launch: items [0, totalA) convert the A_g
@@ -496,12 +506,12 @@ pgk_status launch_quant_fp8_grouped(int transpose, const GQuant* probs, const in
 
 pgk_status launch_cvt_bf16(int rows, int cols, const float* src, int lds, uint16_t* dst, int ldd,
                            int transpose, cudaStream_t st) {
-    return launch_cvt<0>(rows, cols, src, lds, dst, nullptr, ldd, transpose, st);
+    return launch_cvt(0, rows, cols, src, lds, dst, nullptr, ldd, transpose, st);
 }
 
 pgk_status launch_split_bf16(int rows, int cols, const float* src, int lds, uint16_t* hi,
                              uint16_t* lo, int ldd, int transpose, cudaStream_t st) {
-    return launch_cvt<1>(rows, cols, src, lds, hi, lo, ldd, transpose, st);
+    return launch_cvt(1, rows, cols, src, lds, hi, lo, ldd, transpose, st);
 }
 
 }  // namespace pgk

@@ -1751,10 +1751,9 @@ pgk_status tc_gemm_grouped(int G, const pgk_problem* pr, pgk_dtype dtype, const 
     return PGK_OK;
 }
 
-pgk_status launch_cvt_bf16(int rows, int cols, const float* src, int lds, uint16_t* dst, int ldd,
-                           int transpose, cudaStream_t st);
-pgk_status launch_split_bf16(int rows, int cols, const float* src, int lds, uint16_t* hi,
-                             uint16_t* lo, int ldd, int transpose, cudaStream_t st);
+pgk_status launch_cvt_operands(int mode, int M, int N, int K, const float* A, int lda, uint16_t* a0,
+                               uint16_t* a1, const float* B, int ldb, uint16_t* b0, uint16_t* b1, int Kp,
+                               cudaStream_t st);
 pgk_status launch_quant_fp8(int rows, int cols, const float* src, int lds, uint8_t* dst, int ldd,
                             float* scales, int ld_scales, int transpose, cudaStream_t st);
 
@@ -1776,9 +1775,8 @@ static pgk_status tc_gemm_fused(const TcVariant& v, int slices, int M, int N, in
     void* b1 = nullptr;
     if (dtype == PGK_SPLIT_BF16 && !(b1 = workspace(WS_B1, (size_t)N * Kp * 2, &st))) return st;
     if (prep_b) {
-        st = dtype == PGK_SPLIT_BF16
-                 ? launch_split_bf16(K, N, B, ldb, (uint16_t*)b0, (uint16_t*)b1, Kp, 1, s)
-                 : launch_cvt_bf16(K, N, B, ldb, (uint16_t*)b0, Kp, 1, s);
+        st = launch_cvt_operands(dtype == PGK_SPLIT_BF16, M, N, K, nullptr, 0, nullptr, nullptr, B, ldb,
+                                 (uint16_t*)b0, (uint16_t*)b1, Kp, s);
         if (st != PGK_OK) return st;
     }
     TcMaps maps;
@@ -1852,24 +1850,18 @@ pgk_status tc_gemm_fp32_inputs(const pgk_case& c, int M, int N, int K, pgk_dtype
     if (!a0) return st;
     void* b0 = workspace(WS_B0, (size_t)N * Kp * esz, &st);
     if (!b0) return st;
-    if (dtype == PGK_BF16) {
-        if ((st = launch_cvt_bf16(M, K, A, lda, (uint16_t*)a0, Kp, 0, s)) != PGK_OK) return st;
-        if (prep_b && (st = launch_cvt_bf16(K, N, B, ldb, (uint16_t*)b0, Kp, 1, s)) != PGK_OK) return st;
-        return tc_gemm_launch(c, M, N, K, dtype, a0, Kp, b0, Kp, nullptr, nullptr, nullptr, nullptr,
-                              C, ldc, beta, s);
-    }
-    if (dtype == PGK_SPLIT_BF16) {
-        void* a1 = workspace(WS_A1, (size_t)M * Kp * 2, &st);
-        if (!a1) return st;
-        void* b1 = workspace(WS_B1, (size_t)N * Kp * 2, &st);
-        if (!b1) return st;
-        if ((st = launch_split_bf16(M, K, A, lda, (uint16_t*)a0, (uint16_t*)a1, Kp, 0, s)) != PGK_OK)
+    if (dtype != PGK_FP8_E4M3) {
+        const bool split = dtype == PGK_SPLIT_BF16;
+        void* a1 = nullptr;
+        void* b1 = nullptr;
+        if (split) {
+            if (!(a1 = workspace(WS_A1, (size_t)M * Kp * 2, &st))) return st;
+            if (!(b1 = workspace(WS_B1, (size_t)N * Kp * 2, &st))) return st;
+        }
+        if ((st = launch_cvt_operands(split, M, N, K, A, lda, (uint16_t*)a0, (uint16_t*)a1, B, ldb,
+                                      prep_b ? (uint16_t*)b0 : nullptr, (uint16_t*)b1, Kp, s)) != PGK_OK)
             return st;
-        if (prep_b &&
-            (st = launch_split_bf16(K, N, B, ldb, (uint16_t*)b0, (uint16_t*)b1, Kp, 1, s)) != PGK_OK)
-            return st;
-        return tc_gemm_launch(c, M, N, K, dtype, a0, Kp, b0, Kp, a1, b1, nullptr, nullptr, C, ldc,
-                              beta, s);
+        return tc_gemm_launch(c, M, N, K, dtype, a0, Kp, b0, Kp, a1, b1, nullptr, nullptr, C, ldc, beta, s);
     }
     const int mt = (M + 127) / 128, kt = (K + 127) / 128, nt = (N + 127) / 128;
     float* sa = (float*)workspace(WS_SA, (size_t)mt * kt * 4, &st);

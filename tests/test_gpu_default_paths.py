@@ -92,3 +92,29 @@ def test_grouped_wide_tile_on_ragged_problems(dev, shift):
         pgk.gemm(A, B, one, pgk.F32, pgk.params(4, 8, 8, 16, 8))
         assert torch.equal(one, C)
         assert_fp32_gemm(C.cpu().numpy(), A.cpu().numpy(), B.cpu().numpy())
+
+
+@pytest.mark.parametrize("form,prog", [(pgk.SPLIT_BF16, (128, 128, 3, 0, 0)), (pgk.BF16, (128, 256, 4, 0, 0))])
+@pytest.mark.parametrize("M,N,K", [(1, 65, 1), (64, 128, 64), (65, 100, 63), (130, 66, 129), (200, 300, 777)])
+@pytest.mark.parametrize("pad,shift", [(0, 0), (1, 0), (4, 0), (4, 1)])
+def test_both_operands_converted_in_one_launch(dev, form, prog, M, N, K, pad, shift):
+    """The library's conversion of A and B (transposed) in one launch, with strides and
+    bases that allow 128-bit loads and that do not: the product equals the one of
+    operands that the preparation entry points converted, bit for bit."""
+    A, B = (torch.randn(r * (c + pad) + shift, device=dev)[shift:].view(r, c + pad)[:, :c]
+            for r, c in ((M, K), (K, N)))
+    C = torch.full((M, N), float("nan"), device=dev)
+    pgk.gemm(A, B, C, form, pgk.params(*prog))
+    Kp = (K + 15) // 16 * 16
+    a, al, b, bl = (torch.zeros(r, Kp, dtype=torch.int16, device=dev) for r in (M, M, N, N))
+    want = torch.empty(M, N, device=dev)
+    if form == pgk.SPLIT_BF16:
+        pgk.split_bf16(A.contiguous(), a, al, 0)
+        pgk.split_bf16(B.contiguous(), b, bl, 1)
+        pgk.gemm_lowp(M, N, K, form, a, Kp, b, Kp, want, N, A_lo=al, Bt_lo=bl, prog=pgk.params(*prog))
+    else:
+        pgk.cvt_bf16(A.contiguous(), a, 0)
+        pgk.cvt_bf16(B.contiguous(), b, 1)
+        pgk.gemm_lowp(M, N, K, form, a, Kp, b, Kp, want, N, prog=pgk.params(*prog))
+    assert torch.equal(a[:, K:], torch.zeros_like(a[:, K:]))   # entry points write source columns only
+    assert torch.equal(C, want)
