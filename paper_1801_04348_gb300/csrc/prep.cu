@@ -160,6 +160,7 @@ struct CvtOp {
 template <int MODE>
 __global__ void __launch_bounds__(256) k_cvt(const CvtOp a, const CvtOp b) {
     __shared__ float t[64][65];
+    pdl_wait();
     const int i = blockIdx.x;
     if (i < a.items)
         cvt_item<MODE, false>(a.src, a.lds, a.rows, a.cols, a.width, a.vec_in, a.vec_out,
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(256) k_cvt(const CvtOp a, const CvtOp b) {
         cvt_item<MODE, true>(b.src, b.lds, b.rows, b.cols, b.width, b.vec_in, b.vec_out,
                              (i - a.items) / b.item_cols * 64, (i - a.items) % b.item_cols * 64, b.d0, b.d1,
                              b.ldd, t);
+    pdl_trigger();
 }
 
 // Four consecutive elements of row r starting at column c (c a multiple of 4),
@@ -293,9 +295,11 @@ __global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8(int rows, int cols,
                                                              int vec_in, int vec_out) {
     __shared__ float red[QUANT_THREADS / 32];
     __shared__ uint8_t tile[TRANS ? 128 * QUANT_PITCH : 1];
+    pdl_wait();
     quant_tile<TRANS>(src, lds, rows, cols, TRANS ? rows : cols, blockIdx.y * 128, blockIdx.x * 128,
                       dst, ldd, scales + (size_t)blockIdx.y * ld_scales + blockIdx.x, vec_in, vec_out,
                       red, tile);
+    pdl_trigger();
 }
 
 // Grouped quantisation: 128 x 128 tile items over every problem (numbered problem
@@ -313,6 +317,7 @@ __global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8_grouped(const GQuan
                                                                      int ld_scales) {
     __shared__ float red[QUANT_THREADS / 32];
     __shared__ uint8_t tile[TRANS ? 128 * QUANT_PITCH : 1];
+    pdl_wait();
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int g = grouped_item_problem(prefix, G, item);
         const GQuant q = probs[g];
@@ -326,6 +331,7 @@ __global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8_grouped(const GQuan
                           dst + (size_t)q.dst_row * ldd, (int)ldd, so, q.vec, 1, red, tile);
         __syncthreads();   // red is reused by the next item
     }
+    pdl_trigger();
 }
 
 static bool aligned(const void* p, unsigned a) { return ((uintptr_t)p % a) == 0; }
@@ -365,9 +371,7 @@ static pgk_status launch_cvt_ops(int mode, const CvtOp& a, const CvtOp& b, cudaS
         set_error("too many rows for the transposing conversion");
         return PGK_ERR_INVALID_ARG;
     }
-    if (mode == 0) k_cvt<0><<<grid, 256, 0, st>>>(a, b);
-    else k_cvt<1><<<grid, 256, 0, st>>>(a, b);
-    PGK_CUDA_TRY(cudaGetLastError(), "conversion launch");
+    PGK_CUDA_TRY(launch_pdl(mode == 0 ? k_cvt<0> : k_cvt<1>, grid, 256, 0, 1, st, a, b), "conversion launch");
     return PGK_OK;
 }
 
@@ -408,13 +412,9 @@ pgk_status launch_quant_fp8(int rows, int cols, const float* src, int lds, uint8
     }
     const int vec_in = aligned(src, 16) && lds % 4 == 0;
     const int vec_out = aligned(dst, 4) && ldd % 4 == 0;
-    if (transpose)
-        k_quant_fp8<true><<<grid, QUANT_THREADS, 0, st>>>(rows, cols, src, lds, dst, ldd, scales,
-                                                          ld_scales, vec_in, vec_out);
-    else
-        k_quant_fp8<false><<<grid, QUANT_THREADS, 0, st>>>(rows, cols, src, lds, dst, ldd, scales,
-                                                           ld_scales, vec_in, vec_out);
-    PGK_CUDA_TRY(cudaGetLastError(), "FP8 quantisation launch");
+    PGK_CUDA_TRY(launch_pdl(transpose ? k_quant_fp8<true> : k_quant_fp8<false>, grid, QUANT_THREADS, 0, 1, st, rows,
+                            cols, src, lds, dst, ldd, scales, ld_scales, vec_in, vec_out),
+                 "FP8 quantisation launch");
     return PGK_OK;
 }
 
@@ -468,6 +468,7 @@ __global__ void __launch_bounds__(256, 8) k_cvt_grouped(const GCvt* __restrict__
                                                         uint16_t* __restrict__ b0, uint16_t* __restrict__ b1,
                                                         int G, long long ldd) {
     __shared__ float t[64][65];
+    pdl_wait();
     const int item = blockIdx.x;
     if (item < totalA) {
         const int g = warp_item_problem(prefa, G, item);
@@ -476,6 +477,7 @@ __global__ void __launch_bounds__(256, 8) k_cvt_grouped(const GCvt* __restrict__
         const int g = warp_item_problem(prefb, G, item - totalA);
         cvt_grouped_item<MODE, true>(pb[g], item - totalA - __ldg(prefb + g), b0, b1, ldd, t);
     }
+    pdl_trigger();
 }
 
 pgk_status launch_cvt_grouped(int mode, const GCvt* pa, const int* prefa, int totalA, uint16_t* a0,
@@ -487,11 +489,9 @@ pgk_status launch_cvt_grouped(int mode, const GCvt* pa, const int* prefa, int to
         set_error("grouped conversion: too many work items");
         return PGK_ERR_INVALID_ARG;
     }
-    if (mode == 0)
-        k_cvt_grouped<0><<<(unsigned)total, 256, 0, st>>>(pa, prefa, totalA, a0, a1, pb, prefb, b0, b1, G, ldd);
-    else
-        k_cvt_grouped<1><<<(unsigned)total, 256, 0, st>>>(pa, prefa, totalA, a0, a1, pb, prefb, b0, b1, G, ldd);
-    PGK_CUDA_TRY(cudaGetLastError(), "grouped conversion launch");
+    PGK_CUDA_TRY(launch_pdl(mode == 0 ? k_cvt_grouped<0> : k_cvt_grouped<1>, (unsigned)total, 256, 0, 1, st, pa,
+                            prefa, totalA, a0, a1, pb, prefb, b0, b1, G, ldd),
+                 "grouped conversion launch");
     return PGK_OK;
 }
 
@@ -503,13 +503,9 @@ pgk_status launch_quant_fp8_grouped(int transpose, const GQuant* probs, const in
     PGK_CUDA_TRY(cudaGetDevice(&dev), "cudaGetDevice");
     PGK_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
     const int grid = std::min(total, std::max(sms, 1) * 2);
-    if (transpose)
-        k_quant_fp8_grouped<true><<<grid, QUANT_THREADS, 0, st>>>(probs, prefix, G, total, dst, ldd,
-                                                                 scales, ld_scales);
-    else
-        k_quant_fp8_grouped<false><<<grid, QUANT_THREADS, 0, st>>>(probs, prefix, G, total, dst, ldd,
-                                                                  scales, ld_scales);
-    PGK_CUDA_TRY(cudaGetLastError(), "grouped FP8 quantisation launch");
+    PGK_CUDA_TRY(launch_pdl(transpose ? k_quant_fp8_grouped<true> : k_quant_fp8_grouped<false>, (unsigned)grid,
+                            QUANT_THREADS, 0, 1, st, probs, prefix, G, total, dst, ldd, scales, ld_scales),
+                 "grouped FP8 quantisation launch");
     return PGK_OK;
 }
 

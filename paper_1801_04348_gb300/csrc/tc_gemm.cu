@@ -485,6 +485,9 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_sh;
     volatile int* abort_flag = &abort_sh;
+    // the set-up above overlaps the tail of the kernel before (the operand preparation);
+    // from here on its results, the tables and C are read
+    pdl_wait();
 
     // tile t -> (tm, tn): groups of 2048 rows of tiles (16 single-CTA or 8 pair tile
     // rows) walked column by column, so that the tiles resident at once share
@@ -1228,6 +1231,7 @@ __global__ void k_wait_selftest(unsigned int* err, unsigned long long limit_ns) 
 // (deterministic): C = sum_s part[s] (beta = 0) or C += sum_s part[s] (beta = 1).
 __global__ void k_slice_reduce(int M, int N, const float* __restrict__ part, int slices, float* C,
                                int ldc, int beta) {
+    pdl_wait();
     const long long total = (long long)M * N;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
@@ -1325,13 +1329,10 @@ static cudaError_t launch_tc(const TcMaps& maps, const TcParams& p0, long long t
         if (CAN_TAIL) p.tail = tail_tiles(tiles, sm_count, Cfg::BN);
         const int grid = (int)std::min<long long>(tiles + p.tail, sm_count);
         if constexpr (CAN_TAIL) {
-            if (p.tail > 0) {
-                k_tc_gemm<Cfg, false, true><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(maps, p);
-                return cudaGetLastError();
-            }
+            if (p.tail > 0)
+                return launch_pdl(k_tc_gemm<Cfg, false, true>, grid, Cfg::THREADS, Cfg::SMEM, 1, st, maps, p);
         }
-        k_tc_gemm<Cfg, GROUPED><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(maps, p);
-        return cudaGetLastError();
+        return launch_pdl(k_tc_gemm<Cfg, GROUPED>, grid, Cfg::THREADS, Cfg::SMEM, 1, st, maps, p);
     }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1361,11 +1362,11 @@ static cudaError_t launch_tc(const TcMaps& maps, const TcParams& p0, long long t
     clusters = std::min(clusters, sm_count / 2);
     if (CAN_TAIL) p.tail = tail_tiles(tiles, clusters, Cfg::BN);
     clusters = (int)std::min<long long>(tiles + p.tail, clusters);
-    cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
+    const unsigned ctas = 2u * (unsigned)clusters;
     if constexpr (CAN_TAIL) {
-        if (p.tail > 0) return cudaLaunchKernelEx(&cfg, k_tc_gemm<Cfg, false, true>, maps, p);
+        if (p.tail > 0) return launch_pdl(k_tc_gemm<Cfg, false, true>, ctas, Cfg::THREADS, Cfg::SMEM, 2, st, maps, p);
     }
-    return cudaLaunchKernelEx(&cfg, k_tc_gemm<Cfg, GROUPED>, maps, p);
+    return launch_pdl(k_tc_gemm<Cfg, GROUPED>, ctas, Cfg::THREADS, Cfg::SMEM, 2, st, maps, p);
 }
 
 struct TcVariant {
@@ -1824,8 +1825,8 @@ static pgk_status tc_gemm_fused(const TcVariant& v, int slices, int M, int N, in
     if (S > 1) {
         const long long total = (long long)M * N;
         const int blocks = (int)std::min<long long>((total + 255) / 256, (long long)m.sm_count * 8);
-        k_slice_reduce<<<blocks, 256, 0, s>>>(M, N, p.part, S, C, ldc, p.beta);
-        PGK_CUDA_TRY(cudaGetLastError(), "K-slice reduction launch");
+        PGK_CUDA_TRY(launch_pdl(k_slice_reduce, blocks, 256, 0, 1, s, M, N, (const float*)p.part, S, C, ldc, p.beta),
+                     "K-slice reduction launch");
     }
     return PGK_OK;
 }
