@@ -395,27 +395,11 @@ static pgk_status check_gemm_args(int M, int N, int K, const void* A, int lda, c
     return PGK_OK;
 }
 
-// Parameters of a call that names none, for the forms that still take one program
-// (FP32 plans its tile by shape: simt_wide_launch).
-pgk_params default_params(int M, int N, int K, pgk_dtype dtype) {
-    pgk_params p;
-    if (dtype == PGK_I32) {
-        if ((long long)M * N >= 2048LL * 2048) {
-            p.B0 = 16; p.B1 = 16; p.s = 8; p.sr = 8; p.tile = 8;
-        } else if ((long long)M * N >= 256LL * 256) {
-            p.B0 = 16; p.B1 = 16; p.s = 4; p.sr = 4; p.tile = 8;
-        } else {
-            p.B0 = 8; p.B1 = 8; p.s = 8; p.sr = 8; p.tile = 8;
-        }
-        (void)K;
-    } else if (dtype == PGK_SPLIT_BF16) {
-        p.B0 = 128; p.B1 = 128; p.s = 3; p.sr = 0; p.tile = 0;
-    } else if (dtype == PGK_BF16) {
-        p.B0 = 128; p.B1 = 256; p.s = 4; p.sr = 0; p.tile = 0;
-    } else {
-        p.B0 = 128; p.B1 = 128; p.s = 6; p.sr = 0; p.tile = 0;
-    }
-    return p;
+// Parameters of an int32 call that names none (the other forms are planned by shape).
+static pgk_params default_i32_params(int M, int N) {
+    if ((long long)M * N >= 2048LL * 2048) return pgk_params{16, 16, 8, 8, 8};
+    if ((long long)M * N >= 256LL * 256) return pgk_params{16, 16, 4, 4, 8};
+    return pgk_params{8, 8, 8, 8, 8};
 }
 
 }  // namespace pgk
@@ -437,30 +421,32 @@ pgk_status gemm_device(int M, int N, int K, pgk_dtype dtype, const float* A, int
     st = current_machine(&m, NULL);
     if (st != PGK_OK) return st;
     pgk_params p;
-    if (prog) {
-        p = *prog;
-    } else if (pgk_tune_cache_get(M, N, K, dtype, &p) != PGK_OK) {
+    pgk_case c;
+    if (prog || pgk_tune_cache_get(M, N, K, dtype, &p) == PGK_OK) {
+        if (prog) p = *prog;
+        st = select_any(&m, NULL, M, N, K, dtype, &p, &c);
+    } else if ((dtype == PGK_BF16 || dtype == PGK_SPLIT_BF16) && N <= 64 && aligned16(A) && lda % 4 == 0) {
         // skinny products in the BF16 and split forms: the fused-conversion program
         // (A read once, in FP32, by the GEMM) is the leaf of the case discussion
         // whenever N fits its 64-wide tile and A suits TMA; otherwise the learned
-        // selection ranks the tile programs, else the default
-        const bool fused = (dtype == PGK_BF16 || dtype == PGK_SPLIT_BF16) && N <= 64 &&
-                           ((uintptr_t)A & 15u) == 0 && lda % 4 == 0;
-        if (fused) {
-            // sr = 0: the program chooses its K slices for the shape
-            p = pgk_params{128, 64, dtype == PGK_SPLIT_BF16 ? 3 : 4, 0, 0};
-        } else if (learned_select(M, N, K, dtype, A, lda, B, ldb, C, ldc, beta, stream, &p) !=
-                   PGK_OK) {
-            if (dtype == PGK_F32) {
-                const cudaError_t e =
-                    simt_wide_launch(simt_args(M, N, K, A, lda, B, ldb, C, ldc, beta), 0, stream);
-                return e == cudaSuccess ? PGK_OK : cuda_fail(e, "SIMT GEMM launch");
-            }
-            p = default_params(M, N, K, dtype);
-        }
+        // selection ranks the tile programs, else the program is planned for the shape
+        // (sr = 0: this program chooses its K slices for the shape)
+        p = pgk_params{128, 64, dtype == PGK_SPLIT_BF16 ? 3 : 4, 0, 0};
+        st = select_any(&m, NULL, M, N, K, dtype, &p, &c);
+    } else if (learned_select(M, N, K, dtype, A, lda, B, ldb, C, ldc, beta, stream, &p) == PGK_OK) {
+        st = select_any(&m, NULL, M, N, K, dtype, &p, &c);
+    } else if (dtype == PGK_F32) {
+        const cudaError_t e = simt_wide_launch(simt_args(M, N, K, A, lda, B, ldb, C, ldc, beta), 0, stream);
+        return e == cudaSuccess ? PGK_OK : cuda_fail(e, "SIMT GEMM launch");
+    } else if (dtype == PGK_I32) {
+        p = default_i32_params(M, N);
+        st = select_any(&m, NULL, M, N, K, dtype, &p, &c);
+    } else if (dtype == PGK_BF16 || dtype == PGK_SPLIT_BF16 || dtype == PGK_FP8_E4M3) {
+        st = tc_default_case(&m, M, N, K, dtype, &c);
+    } else {
+        set_error("unknown dtype %d", (int)dtype);
+        st = PGK_ERR_INVALID_ARG;
     }
-    pgk_case c;
-    st = select_any(&m, NULL, M, N, K, dtype, &p, &c);
     if (st != PGK_OK) return st;
     if (dtype == PGK_F32 || dtype == PGK_I32)
         return run_simt_case(c, M, N, K, A, lda, B, ldb, C, ldc, beta, stream);

@@ -120,6 +120,8 @@ pgk_status current_machine(pgk_machine* m, int* device);
 // Fills the tensor-core case for (dtype, prog) or returns an error.
 pgk_status tc_select(const pgk_machine* m, int M, int N, int K, pgk_dtype dtype,
                      const pgk_params* prog, pgk_case* out);
+// The case of a call without parameters (program and K slices planned for the shape).
+pgk_status tc_default_case(const pgk_machine* m, int M, int N, int K, pgk_dtype dtype, pgk_case* out);
 pgk_status tc_gemm_launch(const pgk_case& c, int M, int N, int K, pgk_dtype dtype,
                           const void* A, int lda, const void* Bt, int ldbt, const void* A_lo,
                           const void* Bt_lo, const float* sA, const float* sB, float* C, int ldc,

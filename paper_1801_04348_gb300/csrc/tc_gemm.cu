@@ -20,6 +20,8 @@
 // own and only B^T into the stages; the converters write A's BF16 tiles (hi, and
 // lo for split) into the stages.  Their work units may be K slices of a tile,
 // whose partial products k_slice_reduce sums in slice order.
+// A product with few tiles may run each as a cluster of CTAs, one K slice per CTA (KSPLIT):
+// the partial tiles meet in shared memory and every CTA sums a slab of rows over its peers.
 // Every wait is bounded (globaltimer); on timeout the CTA sets the device
 // error word, stops issuing, drains its own TMA and MMA work and frees TMEM.
 //
@@ -36,6 +38,7 @@
 #include <atomic>
 #include <climits>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "pgk_internal.cuh"
@@ -387,7 +390,8 @@ struct TcParams {
     int ntiles_g;
     // fused-conversion programs split over K: work unit t is K slice t % kslices of tile
     // t / kslices (kper K blocks each, the last one shorter); slice s writes its partial
-    // product to part + s M N (row stride N), summed into C by a second launch
+    // product to part + s M N (row stride N), summed into C by a second launch; K-split
+    // launches: slice s is CTA s of the tile's cluster
     int kslices, kper;
     float* part;
 };
@@ -398,9 +402,30 @@ struct TcMaps {
     CUtensorMap a, b, a2, b2, bh, b2h;
 };
 
-// TAIL: the instantiation that runs the last p.tail tiles as column halves; the
-// others compile without any of that logic in their loops.
-template <class Cfg, bool GROUPED = false, bool TAIL = false>
+// shared::cluster load of 16 bytes
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(addr)
+                 : "memory");
+    return v;
+}
+
+// TAIL: the instantiation that runs the last p.tail tiles as column halves; KSPLIT: the one
+// that runs every tile as a cluster of p.kslices K slices.  The others compile without any
+// of that logic in their loops.
+//
+// KSPLIT is for products whose 128 x 128 tiles leave SMs idle: the K loop of a tile, a serial
+// chain of K blocks on one tensor core, is what such a product takes.  A cluster of up to
+// eight CTAs shares it; after its last K block each CTA leaves its FP32 partial tile in its
+// own shared memory (over the stage ring, which is empty then), and after a cluster barrier
+// CTA r sums rows [r, r + 1) 128 / S of all peers through distributed shared memory, in slice
+// order, and stores them: no workspace and no second launch.  Measured per launch on GB300:
+// split 256 x 256 x 4096 39.6 us as four tiles, 11.1 as four clusters of eight; 1024 x 1024 x
+// 8192 76.0 and 43.2 (two slices); 513 x 1030 x 777 11.7 and 10.3 (three); BF16 128 x 128 x
+// 8192 40.5 and 11.4; FP8 1024 x 1024 x 8192 30.4 and 20.1.
+template <class Cfg, bool GROUPED = false, bool TAIL = false, bool KSPLIT = false>
 __global__ void __launch_bounds__(Cfg::THREADS, 1)
     k_tc_gemm(const __grid_constant__ TcMaps tm, TcParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -417,6 +442,9 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
 
     constexpr bool PAIR = Cfg::PAIR;
     static_assert(!(PAIR && GROUPED), "grouped launches use single-CTA tiles");
+    static_assert(!KSPLIT || (!PAIR && !GROUPED && !TAIL && !Cfg::FUSED &&
+                              Cfg::BM * Cfg::BN * 4 <= Cfg::STAGES * Cfg::STAGE_BYTES),
+                  "K-split clusters: single-CTA tiles whose partials fit the stage ring");
     static_assert(!TAIL || (!GROUPED && Cfg::BN == 256 && Cfg::MODE != MODE_FP8),
                   "tail halves: 256-wide single launches of the BF16 and split forms");
     const int warp = threadIdx.x >> 5;
@@ -433,7 +461,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
     const int nfull = tiles_m * tiles_n;
     const int tail = TAIL ? p.tail : 0;
     // work units: every tile, the last `tail` of them twice (one per column half)
-    const int ksl = (Cfg::FUSED && p.kslices > 1) ? p.kslices : 1;
+    const int ksl = ((Cfg::FUSED || KSPLIT) && p.kslices > 1) ? p.kslices : 1;
     const int ntiles = GROUPED ? p.ntiles_g : (nfull + tail) * ksl;
     const int nkb = (p.K + Cfg::BK - 1) / Cfg::BK;
 
@@ -532,7 +560,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             int tt = t;
             ti.half = -1;
             int sl = 0;
-            if (Cfg::FUSED && ksl > 1) {
+            if ((Cfg::FUSED || KSPLIT) && ksl > 1) {
                 sl = t % ksl;
                 tt = t / ksl;
             }
@@ -551,6 +579,10 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             ti.C = p.C;
             ti.kb0 = 0;
             ti.beta = p.beta;
+            if (KSPLIT) {
+                ti.kb0 = sl * p.kper;
+                ti.nkb = min(nkb - ti.kb0, p.kper);
+            }
             if (Cfg::FUSED && ksl > 1) {
                 ti.kb0 = sl * p.kper;
                 ti.nkb = min(nkb - ti.kb0, p.kper);
@@ -664,7 +696,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                         break;
                     }
                     uint8_t* st = tiles + (size_t)stage * Cfg::STAGE_BYTES;
-                    const int x = kb * Cfg::BK;
+                    const int x = (KSPLIT ? ti.kb0 + kb : kb) * Cfg::BK;
                     // passes of MODE_SPLIT3: 0 = (A lo, B hi), 1 = (A hi, B lo), 2 = (A hi, B hi)
                     const CUtensorMap* ma = (Cfg::MODE == MODE_SPLIT3 && v == 0) ? &tm.a2 : &tm.a;
                     const CUtensorMap* mb = (Cfg::MODE == MODE_SPLIT3 && v == 1) ? mbl : mbh;
@@ -1011,6 +1043,15 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             }
             __syncwarp();
         };
+        // K-split: 32 columns from column cb of the tile's rows q 32 .. into this CTA's partial
+        // tile (BN floats a row, the chunks of every 128 bytes swizzled as in the staging)
+        auto stage_partial = [&](const float (&v)[32], int cb) {
+            const int r = q * 32 + lane;
+            float4* d = reinterpret_cast<float4*>(tiles) + (size_t)r * (Cfg::BN / 4) + cb / 4;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                d[j ^ (r & 7)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        };
         const int ncol = Cfg::BN / (Cfg::EPI_WARPS / 4);  // columns handled by this warp
         const int col0 = (e >> 2) * ncol;
         // releases an accumulator: one arrival per warp at the MMA issuer's barrier
@@ -1083,10 +1124,11 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                 // of B^T (both offset by the problem's first block in a grouped launch)
                 const int mblk = ti.rowA / 128 + tm * Cfg::CTAS + (int)pair_rank<PAIR>();
                 const int nblk = ti.rowB / 128 + min(n0 / 128, (tN - 1) / 128);
+                const int cb0 = KSPLIT ? ti.kb0 : 0;   // (FP8 chunks are single K blocks)
                 auto chunk_scale = [&](int c) {
-                    return c < nchunks
-                        ? __ldg(p.sA + (size_t)mblk * ksa + c) * __ldg(p.sB + (size_t)c * nsb + nblk)
-                        : 0.f;
+                    return c < nchunks ? __ldg(p.sA + (size_t)mblk * ksa + cb0 + c) *
+                                             __ldg(p.sB + (size_t)(cb0 + c) * nsb + nblk)
+                                       : 0.f;
                 };
                 float sc_cur = 1.f, sc_nxt = 1.f;
                 if (Cfg::MODE == MODE_FP8) {
@@ -1153,7 +1195,8 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                         v[2 * i] = f2_lo(acc2[g * 16 + i]);
                         v[2 * i + 1] = f2_hi(acc2[g * 16 + i]);
                     }
-                    store_block(v, row0, n0 + g * 32, ti.M, tN, ti.C, ti.ldc, ti.beta);
+                    if (KSPLIT) stage_partial(v, col0 + g * 32);
+                    else store_block(v, row0, n0 + g * 32, ti.M, tN, ti.C, ti.ldc, ti.beta);
                 }
             } else {
                 int w = 1;
@@ -1177,7 +1220,8 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                     float v[32];
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-                    store_block(v, row0, n0 + c * 32, ti.M, tN, ti.C, ti.ldc, ti.beta);
+                    if (KSPLIT) stage_partial(v, col0 + c * 32);
+                    else store_block(v, row0, n0 + c * 32, ti.M, tN, ti.C, ti.ldc, ti.beta);
                 };
                 if (ti.half < 0) {
 #pragma unroll 1
@@ -1196,7 +1240,71 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
     }
 
     tc_fence_before();
-    __syncthreads();
+    if constexpr (KSPLIT) {
+        cluster_sync();   // every partial tile is written (each path to here is bounded)
+        const int S = ksl, rank = (int)blockIdx.x % S;
+        int tmi, tni;
+        coords((int)blockIdx.x / S, tmi, tni);
+        const int rows = (Cfg::BM + S - 1) / S, r_lo = rank * rows, r_n = min(Cfg::BM - r_lo, rows);
+        const uint32_t base = smem_u32(tiles);
+        const bool vec = ((uintptr_t)p.C & 15u) == 0 && (p.ldc & 3) == 0;
+        // NS peers at most; E elements of the slab at a time, so that a thread always has
+        // about eight remote loads in flight (their latency is what the exchange costs)
+        auto reduce = [&](auto ns_c, auto e_c) {
+            constexpr int NS = decltype(ns_c)::value, E = decltype(e_c)::value;
+            for (int i0 = threadIdx.x; i0 < r_n * (Cfg::BN / 4); i0 += E * Cfg::THREADS) {
+                float4 v[E][NS];
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    // (an element beyond the slab reads the first one again)
+                    const int i = i0 + e * Cfg::THREADS < r_n * (Cfg::BN / 4) ? i0 + e * Cfg::THREADS : i0;
+                    const int r = r_lo + i / (Cfg::BN / 4), c4 = i % (Cfg::BN / 4);
+                    const uint32_t a = base + 16u * (uint32_t)(r * (Cfg::BN / 4) + ((c4 & ~7) | ((c4 ^ r) & 7)));
+#pragma unroll
+                    for (int y = 0; y < NS; ++y)
+                        if (y < S) v[e][y] = ld_cluster4(mapa_shared(a, (uint32_t)y));
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int i = i0 + e * Cfg::THREADS;
+                    const int r = r_lo + i / (Cfg::BN / 4), c4 = i % (Cfg::BN / 4);
+                    const int gm = tmi * Cfg::BM + r, gn = tni * Cfg::BN + 4 * c4;
+                    if (i >= r_n * (Cfg::BN / 4) || gm >= p.M || gn >= p.N) continue;
+                    float4 x = v[e][0];
+#pragma unroll
+                    for (int y = 1; y < NS; ++y)
+                        if (y < S) {
+                            x.x += v[e][y].x;
+                            x.y += v[e][y].y;
+                            x.z += v[e][y].z;
+                            x.w += v[e][y].w;
+                        }
+                    float* cp = p.C + (size_t)gm * p.ldc + gn;
+                    if (vec && gn + 3 < p.N) {
+                        if (p.beta) {
+                            const float4 c = *reinterpret_cast<const float4*>(cp);
+                            x = make_float4(c.x + x.x, c.y + x.y, c.z + x.z, c.w + x.w);
+                        }
+                        *reinterpret_cast<float4*>(cp) = x;
+                    } else {
+                        const float o[4] = {x.x, x.y, x.z, x.w};
+                        float c[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) c[u] = p.beta && gn + u < p.N ? cp[u] : 0.f;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (gn + u < p.N) cp[u] = p.beta ? c[u] + o[u] : o[u];
+                    }
+                }
+            }
+        };
+        if (S <= 2) reduce(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
+        else if (S <= 4) reduce(std::integral_constant<int, 4>(), std::integral_constant<int, 2>());
+        else reduce(std::integral_constant<int, 8>(), std::integral_constant<int, 1>());
+        cluster_sync();   // no CTA leaves while a peer may still read its partial tile
+    } else {
+        __syncthreads();
+    }
     // neither CTA of a pair leaves while the other may still arrive on its barriers
     // or the leader's MMAs may still use its shared tiles and tensor memory
     if (PAIR) cluster_sync();
@@ -1369,6 +1477,47 @@ static cudaError_t launch_tc(const TcMaps& maps, const TcParams& p0, long long t
     return launch_pdl(k_tc_gemm<Cfg, GROUPED>, ctas, Cfg::THREADS, Cfg::SMEM, 2, st, maps, p);
 }
 
+// Clusters of `slices` CTAs that can be resident at once (queried once per device and
+// size; 0: none, or the query failed).
+template <class Cfg>
+static int ksplit_clusters(int slices) {
+    static std::atomic<int> resident[64][9];   // clusters + 1
+    int dev = 0;
+    if (slices < 2 || slices > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int c = resident[dev][slices].load();
+    if (c == 0) {
+        const void* fn = (const void*)k_tc_gemm<Cfg, false, false, true>;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)slices;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)slices, 1, 1);
+        cfg.blockDim = dim3(Cfg::THREADS, 1, 1);
+        cfg.dynamicSmemBytes = Cfg::SMEM;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        resident[dev][slices].store(c = n + 1);
+    }
+    return c - 1;
+}
+
+// One cluster of p.kslices CTAs per tile.
+template <class Cfg>
+static cudaError_t launch_ksplit(const TcMaps& maps, const TcParams& p, long long tiles, int, cudaStream_t st) {
+    const cudaError_t e = cudaFuncSetAttribute((const void*)k_tc_gemm<Cfg, false, false, true>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k_tc_gemm<Cfg, false, false, true>, (unsigned)(tiles * p.kslices), Cfg::THREADS, Cfg::SMEM,
+                      (unsigned)p.kslices, st, maps, p);
+}
+
 struct TcVariant {
     int family, BM, BN, stages, smem, threads, tmem_cols;
     int b_box;   // rows of B^T per tensor-map box (per CTA)
@@ -1403,6 +1552,77 @@ static const TcVariant* tc_table(int* n) {
     };
     *n = (int)(sizeof(t) / sizeof(t[0]));
     return t;
+}
+
+// What a tile of each program costs a launch without parameters (us on GB300, at full
+// load): per K block (64 deep, FP8 128) and once per round of tiles.  From the launches
+// alone of 2048^3, 4096^3, 8192^3, 8192 x 1024 x 4096 and 3000 x 3000 x 500; the estimate
+// is within 10 % of them.
+struct TcCost {
+    pgk_dtype dtype;
+    int BM, BN, stages;
+    float block, round;
+    // K-split launch of the same tiles, if there is one
+    int (*clusters)(int slices);
+    tc_launch_fn ksplit;
+};
+template <int MODE, int BN, int ST>
+static TcCost tc_cost(pgk_dtype dtype, float block, float round) {
+    typedef TcCfg<MODE, BN, ST> Cfg;
+    return TcCost{dtype, 128, BN, ST, block, round, ksplit_clusters<Cfg>, launch_ksplit<Cfg>};
+}
+static const TcCost* tc_costs(int* n) {
+    static const TcCost t[] = {
+        tc_cost<MODE_SPLIT, 128, 3>(PGK_SPLIT_BF16, 0.60f, 2.5f),
+        {PGK_SPLIT_BF16, 128, 256, 2, 1.05f, 3.5f, nullptr, nullptr},
+        {PGK_SPLIT_BF16, 256, 256, 3, 0.90f, 7.0f, nullptr, nullptr},
+        tc_cost<MODE_BF16, 128, 6>(PGK_BF16, 0.333f, 2.5f),
+        {PGK_BF16, 128, 256, 4, 0.41f, 3.0f, nullptr, nullptr},
+        {PGK_BF16, 256, 256, 6, 0.34f, 4.5f, nullptr, nullptr},
+        tc_cost<MODE_FP8, 128, 6>(PGK_FP8_E4M3, 0.47f, 2.5f),
+        {PGK_FP8_E4M3, 128, 256, 4, 0.68f, 3.0f, nullptr, nullptr},
+    };
+    *n = (int)(sizeof(t) / sizeof(t[0]));
+    return t;
+}
+
+// The tile program and K slices of a call without parameters: the smallest estimate over
+// the form's programs.  A launch takes ceil(tiles / places) rounds (a last round at most
+// half full runs as column halves in half the time, BF16 and split 256-wide tiles); where
+// 128 x 128 tiles leave places idle, clusters of 2 to 8 K slices (as many as can be resident
+// at once: 76 of two, 15 of eight) share their K blocks at 3 us for the exchange.  Against one fixed program per form: split 8192^3 2020 -> 1630 us a
+// launch (CTA pairs), FP8 8192 x 1024 x 4096 66 -> 49 (256-wide tiles).
+static void tc_plan(const pgk_machine& m, int M, int N, int K, pgk_dtype dtype, pgk_params* p, int* slices) {
+    int n;
+    const TcCost* t = tc_costs(&n);
+    const int nkb = (int)(((long long)K + (dtype == PGK_FP8_E4M3 ? 127 : 63)) / (dtype == PGK_FP8_E4M3 ? 128 : 64));
+    double best = 0;
+    bool any = false;
+    for (int i = 0; i < n; ++i) {
+        if (t[i].dtype != dtype) continue;
+        const long long tiles =
+            (((long long)M + t[i].BM - 1) / t[i].BM) * (((long long)N + t[i].BN - 1) / t[i].BN);
+        const long long places = t[i].BM == 256 ? m.sm_count / 2 : m.sm_count;
+        const long long rem = tiles % places;
+        double rounds = (double)((tiles + places - 1) / places);
+        if (t[i].BN == 256 && dtype != PGK_FP8_E4M3 && rem > 0 && 2 * rem <= places) rounds -= 0.5;
+        const double est = rounds * (nkb * t[i].block + t[i].round);
+        if (!any || est < best) {
+            any = true;
+            best = est;
+            *p = pgk_params{t[i].BM, t[i].BN, t[i].stages, 0, 0};
+            *slices = 1;
+        }
+        if (!t[i].clusters) continue;
+        for (int s = 2; s <= 8 && s <= nkb && tiles * s <= m.sm_count; ++s) {
+            const int kper = (nkb + s - 1) / s;
+            const double es = kper * t[i].block + t[i].round + 3.0;
+            if (es >= best || (nkb + kper - 1) / kper != s || tiles > t[i].clusters(s)) continue;
+            best = es;
+            *p = pgk_params{t[i].BM, t[i].BN, t[i].stages, 0, 0};
+            *slices = s;
+        }
+    }
 }
 
 static int tc_base_id = -1;  // registry index of the first tensor-core variant
@@ -1489,6 +1709,16 @@ pgk_status tc_select(const pgk_machine* m, int M, int N, int K, pgk_dtype dtype,
     return PGK_ERR_UNSUPPORTED;
 }
 
+// The case of a call without parameters: tc_plan's program, its K slices in params.sr.
+pgk_status tc_default_case(const pgk_machine* m, int M, int N, int K, pgk_dtype dtype, pgk_case* out) {
+    pgk_params p;
+    int slices = 1;
+    tc_plan(*m, M, N, K, dtype, &p, &slices);
+    const pgk_status st = tc_select(m, M, N, K, dtype, &p, out);
+    if (st == PGK_OK && slices > 1) out->params.sr = slices;
+    return st;
+}
+
 pgk_status tc_gemm_launch(const pgk_case& c, int M, int N, int K, pgk_dtype dtype, const void* A,
                           int lda, const void* Bt, int ldbt, const void* A_lo, const void* Bt_lo,
                           const float* sA, const float* sB, float* C, int ldc, int beta,
@@ -1543,7 +1773,21 @@ pgk_status tc_gemm_launch(const pgk_case& c, int M, int N, int K, pgk_dtype dtyp
     p.err = device_error_word(&st);
     if (!p.err) return st;
     const long long tiles = (long long)((M + t[i].BM - 1) / t[i].BM) * ((N + t[i].BN - 1) / t[i].BN);
-    cudaError_t e = t[i].launch(maps, p, tiles, m.sm_count, stream);
+    tc_launch_fn launch = t[i].launch;
+    if (c.params.sr > 1) {
+        // planned K slices of a tile program (tc_default_case)
+        int nc;
+        const TcCost* k = tc_costs(&nc);
+        for (int j = 0; j < nc; ++j)
+            if (k[j].dtype == dtype && k[j].BM == t[i].BM && k[j].BN == t[i].BN && k[j].stages == t[i].stages &&
+                k[j].ksplit) {
+                const int nkb = (K + (esz == 1 ? 127 : 63)) / (esz == 1 ? 128 : 64);
+                launch = k[j].ksplit;
+                p.kslices = c.params.sr;
+                p.kper = (nkb + p.kslices - 1) / p.kslices;
+            }
+    }
+    cudaError_t e = launch(maps, p, tiles, m.sm_count, stream);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core GEMM launch");
     return PGK_OK;
 }
@@ -1896,15 +2140,9 @@ extern "C" pgk_status pgk_gemm_lowp(int M, int N, int K, pgk_dtype dtype, const 
     pgk_status st = current_machine(&m, NULL);
     if (st != PGK_OK) return st;
     pgk_params p;
-    if (prog) {
-        p = *prog;
-    } else if (pgk_tune_cache_get(M, N, K, dtype, &p) != PGK_OK) {
-        pgk_params d = {128, dtype == PGK_SPLIT_BF16 ? 128 : (dtype == PGK_BF16 ? 256 : 128),
-                        dtype == PGK_SPLIT_BF16 ? 3 : (dtype == PGK_BF16 ? 4 : 6), 0, 0};
-        p = d;
-    }
     pgk_case c;
-    st = tc_select(&m, M, N, K, dtype, &p, &c);
+    if (!prog && pgk_tune_cache_get(M, N, K, dtype, &p) == PGK_OK) prog = &p;
+    st = prog ? tc_select(&m, M, N, K, dtype, prog, &c) : tc_default_case(&m, M, N, K, dtype, &c);
     if (st != PGK_OK) return st;
     return tc_gemm_launch(c, M, N, K, dtype, A, lda, Bt, ldbt, A_lo, Bt_lo, scaleA, scaleB, C, ldc,
                           beta, (cudaStream_t)stream);

@@ -118,3 +118,27 @@ def test_both_operands_converted_in_one_launch(dev, form, prog, M, N, K, pad, sh
         pgk.gemm_lowp(M, N, K, form, a, Kp, b, Kp, want, N, prog=pgk.params(*prog))
     assert torch.equal(a[:, K:], torch.zeros_like(a[:, K:]))   # entry points write source columns only
     assert torch.equal(C, want)
+
+
+@pytest.mark.parametrize("form", [pgk.SPLIT_BF16, pgk.BF16, pgk.FP8_E4M3])
+@pytest.mark.parametrize("M,N,K", [(1, 65, 513), (128, 128, 128), (129, 65, 4096), (200, 300, 1000), (513, 1030, 777),
+                                   (130, 129, 8200), (256, 2048, 640), (2050, 1030, 200), (4000, 3000, 100)])
+@pytest.mark.parametrize("pad,beta", [(0, 0), (5, 1), (4, 1)])
+def test_planned_tensor_core_program(dev, form, M, N, K, pad, beta):
+    """Products without parameters on the planned program: clusters of K slices where the
+    tiles are few (ragged edges, slices of unequal depth, more CTAs than K blocks), CTA
+    pairs and wide tiles where they are many.  Small integers (FP8: a 7 in every 128 x 128
+    tile makes its scale 2^-6) keep every product and sum exact, so the result equals
+    binary64's; nothing beyond column N is written."""
+    g = torch.Generator(device=dev).manual_seed(M + N + K)
+    A, B, C0 = (torch.randint(-7, 8, (r, c + pad), generator=g, device=dev).float()[:, :c]
+                for r, c in ((M, K), (K, N), (M, N)))
+    A[::128, ::128] = B[::128, ::128] = 7
+    C = torch.full((M, N + pad), float("nan"), device=dev)
+    C[:, :N] = C0
+    pgk.gemm(A, B, C[:, :N], form, beta=beta)
+    torch.cuda.synchronize()
+    pgk.check_device_error()
+    want = A.double() @ B.double() + (C0.double() if beta else 0)
+    assert torch.equal(C[:, :N].double(), want)
+    assert torch.isnan(C[:, N:]).all()
