@@ -79,6 +79,28 @@ pgk_status current_machine(pgk_machine* m, int* device) {
     return query_machine(dev, m);
 }
 
+// ------------------------------------------------------ shared-memory limits
+static std::atomic<unsigned> g_smem_epoch{1};
+
+cudaError_t allow_smem(SmemLimit& limit, const void* kernel, int bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned now = g_smem_epoch.load();
+    if (limit.epoch.load() != now) {
+        limit.devices.store(0);
+        limit.epoch.store(now);
+    }
+    const uint64_t bit = 1ull << (dev & 63);
+    if (dev < 64 && (limit.devices.load() & bit)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && dev < 64) limit.devices.fetch_or(bit);
+    return e;
+}
+
+void smem_limits_release() { g_smem_epoch.fetch_add(1); }
+
 // --------------------------------------------------------- variant registry
 static std::vector<Variant> g_registry;
 static bool g_registry_init = false;
@@ -556,6 +578,7 @@ pgk_status pgk_shutdown(void) {
     hostio_release();
     tune_cache_release();
     noalloc_release();
+    smem_limits_release();
     free_workspaces();
     return PGK_OK;
 }

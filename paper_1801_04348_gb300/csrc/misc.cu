@@ -5,9 +5,11 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "pgk_internal.cuh"
@@ -118,20 +120,36 @@ void free_workspaces() {
 }
 
 // ------------------------------------------------------------ tuning cache
+// Keyed by an interned device tag ("<name>_sm<cc>") and the shape; a lookup formats nothing
+// and, while the cache is empty, takes no lock.
+struct TuneKey {
+    int tag, M, N, K, dtype;
+    bool operator<(const TuneKey& o) const {
+        return std::tie(tag, M, N, K, dtype) < std::tie(o.tag, o.M, o.N, o.K, o.dtype);
+    }
+};
 static std::mutex g_tc_mu;
-static std::map<std::string, pgk_params> g_tune;
+static std::vector<std::string> g_tags;   // interned device tags, never removed
+static std::map<TuneKey, pgk_params> g_tune;
+static std::atomic<size_t> g_tune_size{0};
 
-// Device part of the cache key ("<name>_sm<cc>"), looked up once per device.
-static std::string device_tag() {
-    static std::mutex mu;
-    static std::string tags[64];
+// (with g_tc_mu held)
+static int intern_tag(const std::string& tag) {
+    for (size_t i = 0; i < g_tags.size(); ++i)
+        if (g_tags[i] == tag) return (int)i;
+    g_tags.push_back(tag);
+    return (int)g_tags.size() - 1;
+}
+
+// Device part of the cache key, looked up once per device (with g_tc_mu held).
+static int device_tag() {
+    static int tags[64];   // tag + 1
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
         cudaGetLastError();
-        return "unknown";
+        return intern_tag("unknown");
     }
-    std::lock_guard<std::mutex> lk(mu);
-    if (tags[dev].empty()) {
+    if (tags[dev] == 0) {
         cudaDeviceProp p;
         char name[300] = "unknown";
         if (cudaGetDeviceProperties(&p, dev) == cudaSuccess) {
@@ -141,20 +159,15 @@ static std::string device_tag() {
         }
         for (char* c = name; *c; ++c)
             if (*c == ' ' || *c == '\t') *c = '_';
-        tags[dev] = name;
+        tags[dev] = intern_tag(name) + 1;
     }
-    return tags[dev];
-}
-
-static std::string tune_key(int M, int N, int K, pgk_dtype dtype) {
-    char buf[512];
-    snprintf(buf, sizeof(buf), "%s %d %d %d %d", device_tag().c_str(), M, N, K, (int)dtype);
-    return buf;
+    return tags[dev] - 1;
 }
 
 void tune_cache_release() {
     std::lock_guard<std::mutex> lk(g_tc_mu);
     g_tune.clear();
+    g_tune_size.store(0);
 }
 
 // -------------------------------------------------------- default candidates
@@ -380,9 +393,9 @@ pgk_status pgk_tune_cache_put(int M, int N, int K, pgk_dtype dtype, const pgk_pa
         set_error("NULL params");
         return PGK_ERR_INVALID_ARG;
     }
-    const std::string k = tune_key(M, N, K, dtype);
     std::lock_guard<std::mutex> lk(g_tc_mu);
-    g_tune[k] = *p;
+    g_tune[TuneKey{device_tag(), M, N, K, (int)dtype}] = *p;
+    g_tune_size.store(g_tune.size());
     return PGK_OK;
 }
 
@@ -391,9 +404,9 @@ pgk_status pgk_tune_cache_get(int M, int N, int K, pgk_dtype dtype, pgk_params* 
         set_error("NULL params");
         return PGK_ERR_INVALID_ARG;
     }
-    const std::string k = tune_key(M, N, K, dtype);
+    if (g_tune_size.load() == 0) return PGK_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(g_tc_mu);
-    std::map<std::string, pgk_params>::iterator it = g_tune.find(k);
+    const auto it = g_tune.find(TuneKey{device_tag(), M, N, K, (int)dtype});
     if (it == g_tune.end()) return PGK_ERR_INVALID_ARG;
     *p = it->second;
     return PGK_OK;
@@ -411,9 +424,9 @@ pgk_status pgk_tune_cache_save(const char* path) {
     }
     std::lock_guard<std::mutex> lk(g_tc_mu);
     fprintf(f, "# pgk tuning cache v1: device M N K dtype B0 B1 s sr tile\n");
-    for (std::map<std::string, pgk_params>::iterator it = g_tune.begin(); it != g_tune.end(); ++it)
-        fprintf(f, "%s %d %d %d %d %d\n", it->first.c_str(), it->second.B0, it->second.B1,
-                it->second.s, it->second.sr, it->second.tile);
+    for (const auto& e : g_tune)
+        fprintf(f, "%s %d %d %d %d %d %d %d %d %d\n", g_tags[e.first.tag].c_str(), e.first.M, e.first.N,
+                e.first.K, e.first.dtype, e.second.B0, e.second.B1, e.second.s, e.second.sr, e.second.tile);
     fclose(f);
     return PGK_OK;
 }
@@ -437,11 +450,10 @@ pgk_status pgk_tune_cache_load(const char* path) {
         pgk_params p;
         if (sscanf(line, "%511s %d %d %d %d %d %d %d %d %d", dev, &M, &N, &K, &dt, &p.B0, &p.B1,
                    &p.s, &p.sr, &p.tile) == 10) {
-            char key[800];
-            snprintf(key, sizeof(key), "%s %d %d %d %d", dev, M, N, K, dt);
-            g_tune[key] = p;
+            g_tune[TuneKey{intern_tag(dev), M, N, K, dt}] = p;
         }
     }
+    g_tune_size.store(g_tune.size());
     fclose(f);
     return PGK_OK;
 }

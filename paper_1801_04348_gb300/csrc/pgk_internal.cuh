@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -85,6 +86,16 @@ cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, unsigned threads, s
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+
+// The dynamic shared memory a kernel may take beyond 48 KiB, set once per kernel and device
+// instead of on every launch (about 0.4 us each).  pgk_shutdown() forgets what was set: a
+// device reset after it gives the kernels their first limits back.
+struct SmemLimit {
+    std::atomic<uint64_t> devices{0};   // one bit per device
+    std::atomic<unsigned> epoch{0};
+};
+cudaError_t allow_smem(SmemLimit& limit, const void* kernel, int bytes);
+void smem_limits_release();
 
 // Registration hooks, one per translation unit that defines variants.
 void register_simt_variants(std::vector<Variant>& v);

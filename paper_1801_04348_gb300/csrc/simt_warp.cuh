@@ -292,11 +292,10 @@ static cudaError_t launch_wt(const SimtArgs& p, int groups, float* P, cudaStream
     const long long kper = std::min<long long>(
         INT_MAX, ((p.K + (long long)slices - 1) / slices + Cfg::BK - 1) / Cfg::BK * Cfg::BK);
     const bool vec = wt_vec(p.vecA, p.vecB, p.N, p.K);
-    const void* f = vec ? (const void*)k_wt<Cfg, true> : (const void*)k_wt<Cfg, false>;
-    if (Cfg::SMEM > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-        if (e != cudaSuccess) return e;
-    }
+    static SmemLimit limit[2];
+    const cudaError_t e = allow_smem(limit[vec], vec ? (const void*)k_wt<Cfg, true> : (const void*)k_wt<Cfg, false>,
+                                     Cfg::SMEM);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)tiles, (unsigned)groups);
     if (vec) k_wt<Cfg, true><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);
     else k_wt<Cfg, false><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);

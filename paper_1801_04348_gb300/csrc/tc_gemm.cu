@@ -1419,7 +1419,8 @@ template <class Cfg, bool GROUPED>
 static cudaError_t launch_tc(const TcMaps& maps, const TcParams& p0, long long tiles, int sm_count,
                              cudaStream_t st) {
     const void* fn = (const void*)k_tc_gemm<Cfg, GROUPED>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+    static SmemLimit limit;
+    cudaError_t e = allow_smem(limit, fn, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     TcParams p = p0;
     p.tail = 0;
@@ -1430,8 +1431,8 @@ static cudaError_t launch_tc(const TcMaps& maps, const TcParams& p0, long long t
     const void* fn_tail = fn;
     if constexpr (CAN_TAIL) {
         fn_tail = (const void*)k_tc_gemm<Cfg, false, true>;
-        e = cudaFuncSetAttribute(fn_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-        if (e != cudaSuccess) return e;
+        static SmemLimit limit_tail;
+        if ((e = allow_smem(limit_tail, fn_tail, Cfg::SMEM)) != cudaSuccess) return e;
     }
     if (!Cfg::PAIR) {
         if (CAN_TAIL) p.tail = tail_tiles(tiles, sm_count, Cfg::BN);
@@ -1511,8 +1512,8 @@ static int ksplit_clusters(int slices) {
 // One cluster of p.kslices CTAs per tile.
 template <class Cfg>
 static cudaError_t launch_ksplit(const TcMaps& maps, const TcParams& p, long long tiles, int, cudaStream_t st) {
-    const cudaError_t e = cudaFuncSetAttribute((const void*)k_tc_gemm<Cfg, false, false, true>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
+    static SmemLimit limit;
+    const cudaError_t e = allow_smem(limit, (const void*)k_tc_gemm<Cfg, false, false, true>, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_tc_gemm<Cfg, false, false, true>, (unsigned)(tiles * p.kslices), Cfg::THREADS, Cfg::SMEM,
                       (unsigned)p.kslices, st, maps, p);
@@ -1740,7 +1741,10 @@ pgk_status tc_gemm_launch(const pgk_case& c, int M, int N, int K, pgk_dtype dtyp
     TcMaps maps;
     if ((st = make_map(&maps.a, A, M, K, lda, esz, 128)) != PGK_OK) return st;
     if ((st = make_map(&maps.b, Bt, N, K, ldbt, esz, t[i].b_box)) != PGK_OK) return st;
-    if ((st = make_map(&maps.bh, Bt, N, K, ldbt, esz, t[i].b_box / 2)) != PGK_OK) return st;
+    // half-height boxes of B^T: only the 256-wide BF16 and split tiles have column halves
+    const bool halves = t[i].BN == 256 && dtype != PGK_FP8_E4M3;
+    maps.bh = maps.b;
+    if (halves && (st = make_map(&maps.bh, Bt, N, K, ldbt, esz, t[i].b_box / 2)) != PGK_OK) return st;
     if (dtype == PGK_SPLIT_BF16) {
         if (!A_lo || !Bt_lo) {
             set_error("split form needs the lo operands");
@@ -1748,7 +1752,8 @@ pgk_status tc_gemm_launch(const pgk_case& c, int M, int N, int K, pgk_dtype dtyp
         }
         if ((st = make_map(&maps.a2, A_lo, M, K, lda, esz, 128)) != PGK_OK) return st;
         if ((st = make_map(&maps.b2, Bt_lo, N, K, ldbt, esz, t[i].b_box)) != PGK_OK) return st;
-        if ((st = make_map(&maps.b2h, Bt_lo, N, K, ldbt, esz, t[i].b_box / 2)) != PGK_OK) return st;
+        maps.b2h = maps.b2;
+        if (halves && (st = make_map(&maps.b2h, Bt_lo, N, K, ldbt, esz, t[i].b_box / 2)) != PGK_OK) return st;
     } else {
         maps.a2 = maps.a;
         maps.b2 = maps.b;

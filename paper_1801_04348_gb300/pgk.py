@@ -160,10 +160,27 @@ def _ptr(x):
     return x.data_ptr()
 
 
+_raw_stream = None   # () -> handle of torch's current stream on the current device
+
+
+def _current_stream():
+    """torch's current stream as a raw handle, without building a Stream object per call
+    where this torch offers that."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()   # initialises CUDA
+        dev, raw = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if dev is not None and raw is not None:
+            _raw_stream = lambda: raw(dev())   # noqa: E731
+        else:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream   # noqa: E731
+    return _raw_stream()
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
