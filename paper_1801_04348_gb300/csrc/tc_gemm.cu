@@ -412,6 +412,12 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
     return v;
 }
 
+__device__ __forceinline__ float ld_cluster1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
 // TAIL: the instantiation that runs the last p.tail tiles as column halves; KSPLIT: the one
 // that runs every tile as a cluster of p.kslices K slices.  The others compile without any
 // of that logic in their loops.
@@ -1248,59 +1254,86 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
         const int rows = (Cfg::BM + S - 1) / S, r_lo = rank * rows, r_n = min(Cfg::BM - r_lo, rows);
         const uint32_t base = smem_u32(tiles);
         const bool vec = ((uintptr_t)p.C & 15u) == 0 && (p.ldc & 3) == 0;
-        // NS peers at most; E elements of the slab at a time, so that a thread always has
-        // about eight remote loads in flight (their latency is what the exchange costs)
-        auto reduce = [&](auto ns_c, auto e_c) {
+        // A warp takes a row at a time (BN = 128: one 16-byte chunk per lane, or, where C's
+        // rows are not 16-byte aligned, four columns 32 apart, so that C is still accessed
+        // along its rows).  NS peers at most, E rows at a time: a thread always has about
+        // eight remote loads, and with beta = 1 its part of C, in flight together (their
+        // latency is what the exchange costs).
+        static_assert(!KSPLIT || Cfg::BN == 128, "a warp covers a row of the partial tile");
+        auto reduce = [&](auto ns_c, auto e_c, auto vec_c) {
             constexpr int NS = decltype(ns_c)::value, E = decltype(e_c)::value;
-            for (int i0 = threadIdx.x; i0 < r_n * (Cfg::BN / 4); i0 += E * Cfg::THREADS) {
-                float4 v[E][NS];
+            constexpr bool VEC = decltype(vec_c)::value;
+            constexpr int NW = Cfg::THREADS / 32;
+            const int n0 = tni * Cfg::BN;
+            for (int i0 = warp; i0 < r_n; i0 += E * NW) {
+                float4 v[E][NS], c[E];
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    // (an element beyond the slab reads the first one again)
-                    const int i = i0 + e * Cfg::THREADS < r_n * (Cfg::BN / 4) ? i0 + e * Cfg::THREADS : i0;
-                    const int r = r_lo + i / (Cfg::BN / 4), c4 = i % (Cfg::BN / 4);
-                    const uint32_t a = base + 16u * (uint32_t)(r * (Cfg::BN / 4) + ((c4 & ~7) | ((c4 ^ r) & 7)));
+                    // (a row beyond the slab reads its first one again)
+                    const int r = r_lo + (i0 + e * NW < r_n ? i0 + e * NW : i0);
+                    const uint32_t a = base + 512u * (uint32_t)r;
+                    if (VEC) {
 #pragma unroll
-                    for (int y = 0; y < NS; ++y)
-                        if (y < S) v[e][y] = ld_cluster4(mapa_shared(a, (uint32_t)y));
+                        for (int y = 0; y < NS; ++y)
+                            if (y < S)
+                                v[e][y] = ld_cluster4(mapa_shared(
+                                    a + 16u * (uint32_t)((lane & ~7) | ((lane ^ r) & 7)), (uint32_t)y));
+                    } else {
+                        // column 32 u + lane: chunk 8 u + lane / 4 of the row
+                        const uint32_t o = a + 16u * (uint32_t)(((lane >> 2) ^ r) & 7) + 4u * (lane & 3);
+#pragma unroll
+                        for (int y = 0; y < NS; ++y)
+                            if (y < S) {
+                                const uint32_t q = mapa_shared(o, (uint32_t)y);
+                                v[e][y] = make_float4(ld_cluster1(q), ld_cluster1(q + 128u),
+                                                      ld_cluster1(q + 256u), ld_cluster1(q + 384u));
+                            }
+                    }
+                    if (p.beta) {
+                        const int gm = tmi * Cfg::BM + r;
+                        const float* cp = p.C + (size_t)gm * p.ldc + n0;
+                        const int n = gm < p.M ? p.N - n0 : 0;   // columns of this row in C
+                        if (VEC && 4 * lane + 3 < n) {
+                            c[e] = *reinterpret_cast<const float4*>(cp + 4 * lane);
+                        } else {
+                            constexpr int F = VEC ? 4 : 1, U = VEC ? 1 : 32;
+                            c[e] = make_float4(F * lane < n ? cp[F * lane] : 0.f,
+                                               F * lane + U < n ? cp[F * lane + U] : 0.f,
+                                               F * lane + 2 * U < n ? cp[F * lane + 2 * U] : 0.f,
+                                               F * lane + 3 * U < n ? cp[F * lane + 3 * U] : 0.f);
+                        }
+                    }
                 }
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    const int i = i0 + e * Cfg::THREADS;
-                    const int r = r_lo + i / (Cfg::BN / 4), c4 = i % (Cfg::BN / 4);
-                    const int gm = tmi * Cfg::BM + r, gn = tni * Cfg::BN + 4 * c4;
-                    if (i >= r_n * (Cfg::BN / 4) || gm >= p.M || gn >= p.N) continue;
+                    const int gm = tmi * Cfg::BM + r_lo + i0 + e * NW;
+                    if (i0 + e * NW >= r_n || gm >= p.M) continue;
                     float4 x = v[e][0];
 #pragma unroll
                     for (int y = 1; y < NS; ++y)
-                        if (y < S) {
-                            x.x += v[e][y].x;
-                            x.y += v[e][y].y;
-                            x.z += v[e][y].z;
-                            x.w += v[e][y].w;
-                        }
-                    float* cp = p.C + (size_t)gm * p.ldc + gn;
-                    if (vec && gn + 3 < p.N) {
-                        if (p.beta) {
-                            const float4 c = *reinterpret_cast<const float4*>(cp);
-                            x = make_float4(c.x + x.x, c.y + x.y, c.z + x.z, c.w + x.w);
-                        }
-                        *reinterpret_cast<float4*>(cp) = x;
+                        if (y < S) x = make_float4(x.x + v[e][y].x, x.y + v[e][y].y, x.z + v[e][y].z, x.w + v[e][y].w);
+                    if (p.beta) x = make_float4(c[e].x + x.x, c[e].y + x.y, c[e].z + x.z, c[e].w + x.w);
+                    float* cp = p.C + (size_t)gm * p.ldc + n0;
+                    const int n = p.N - n0;
+                    if (VEC && 4 * lane + 3 < n) {
+                        *reinterpret_cast<float4*>(cp + 4 * lane) = x;
                     } else {
-                        const float o[4] = {x.x, x.y, x.z, x.w};
-                        float c[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) c[u] = p.beta && gn + u < p.N ? cp[u] : 0.f;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            if (gn + u < p.N) cp[u] = p.beta ? c[u] + o[u] : o[u];
+                        constexpr int F = VEC ? 4 : 1, U = VEC ? 1 : 32;
+                        if (F * lane < n) cp[F * lane] = x.x;
+                        if (F * lane + U < n) cp[F * lane + U] = x.y;
+                        if (F * lane + 2 * U < n) cp[F * lane + 2 * U] = x.z;
+                        if (F * lane + 3 * U < n) cp[F * lane + 3 * U] = x.w;
                     }
                 }
             }
         };
-        if (S <= 2) reduce(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
-        else if (S <= 4) reduce(std::integral_constant<int, 4>(), std::integral_constant<int, 2>());
-        else reduce(std::integral_constant<int, 8>(), std::integral_constant<int, 1>());
+        auto by_size = [&](auto vec_c) {
+            if (S <= 2) reduce(std::integral_constant<int, 2>(), std::integral_constant<int, 4>(), vec_c);
+            else if (S <= 4) reduce(std::integral_constant<int, 4>(), std::integral_constant<int, 2>(), vec_c);
+            else reduce(std::integral_constant<int, 8>(), std::integral_constant<int, 1>(), vec_c);
+        };
+        if (vec) by_size(std::true_type());
+        else by_size(std::false_type());
         cluster_sync();   // no CTA leaves while a peer may still read its partial tile
     } else {
         __syncthreads();
