@@ -4,10 +4,11 @@
 // FP32 vector: W1 (64x7), b1 (64), W2 (64x64), b2 (64), w3 (64), b3.
 //
 //  * forward: one thread per sample, weights staged in shared memory;
-//  * loss + gradient: one block per 16-sample tile computes the forward pass,
-//    the mean-squared-error gradient and the back-propagated parameter
-//    gradient of its tile in shared memory, writes a per-tile partial; a second
-//    kernel sums the partials in tile order (deterministic);
+//  * loss + gradient: blocks compute the forward pass, the mean-squared-error
+//    gradient and the back-propagated parameter gradient of tiles of 2 to 16
+//    samples in shared memory and add them up in registers; each writes one
+//    partial, and a second kernel sums the partials in a fixed order
+//    (deterministic);
 //  * Adam: elementwise update with host-computed bias corrections.
 #include <math.h>
 
@@ -23,8 +24,8 @@ static constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + H * D_IN, OFF_W2 = OFF_B1 + H
                      OFF_B2 = OFF_W2 + H * H, OFF_W3 = OFF_B2 + H, OFF_B3 = OFF_W3 + H,
                      NPARAM = OFF_B3 + 1;
 static_assert(NPARAM == PGK_MLP_PARAMS, "parameter packing");
-static constexpr int TILE = 16;          // samples per gradient block
 static constexpr int GTHREADS = 256;
+static constexpr int GRAD_BLOCKS = 304;   // most partials of a gradient (two blocks an SM)
 
 __global__ void __launch_bounds__(128) k_mlp_forward(int n, const float* __restrict__ X,
                                                      const float* __restrict__ theta,
@@ -55,142 +56,220 @@ __global__ void __launch_bounds__(128) k_mlp_forward(int n, const float* __restr
     y[s] = out;
 }
 
-// Per-tile forward + backward.  partial[tile][NPARAM + 1]: gradient of
-// (1/n) sum (y - t)^2 restricted to the tile's samples, then the tile's sum of
-// squared residuals.
+// Samples per tile: small batches spread over at most 128 blocks (the partials that the
+// allocation-free entry point holds for its 2048 samples), larger ones take 16.
+static int grad_tile(int n) { return n <= 256 ? 2 : n <= 512 ? 4 : n <= 1024 ? 8 : 16; }
+static int grad_partials(int n) {
+    const int t = grad_tile(n);
+    return std::min((n + t - 1) / t, GRAD_BLOCKS);
+}
+
+// Forward + backward of tiles blockIdx.x, blockIdx.x + gridDim.x, ...  partial[block]
+// [NPARAM + 1]: the gradient of (1/n) sum (y - t)^2 restricted to the block's samples, then
+// their sum of squared residuals.
+//
+// Bound by latency: a minibatch of 256 is 7 MFLOP.  W2 sits in shared memory with a pitch of
+// 65 words, so that a warp reads it without conflicts along either index (with a pitch of
+// 64 the 32 outputs of a warp met in one bank); a thread computes one unit of up to four
+// samples and reads a weight once for all of them, and owns 4 x 4 entries of dW2, two of dW1
+// and one bias or w3 entry, summed in registers over its tiles.  256 samples ran as 16 blocks
+// of 16 samples, 28 us under the profiler; a training step (gradient, sum, Adam) of 128 blocks of
+// two samples, the three launches overlapping, takes 14.6 us instead of 34.8.
+template <int TILE>
 __global__ void __launch_bounds__(GTHREADS) k_mlp_grad_tile(int n, const int* __restrict__ idx,
                                                            const float* __restrict__ X,
                                                            const float* __restrict__ T,
                                                            const float* __restrict__ theta,
                                                            float* __restrict__ partial) {
-    __shared__ float w[NPARAM];
-    __shared__ float xs[TILE][D_IN];
-    __shared__ float z1[TILE][H + 1];
-    __shared__ float z2[TILE][H + 1];
-    __shared__ float d2[TILE][H + 1];   // dL/dz2
-    __shared__ float d1[TILE][H + 1];   // dL/dz1
-    __shared__ float dy[TILE];
-    __shared__ float red[GTHREADS / 32];
-    const int tid = threadIdx.x;
-    const int s0 = blockIdx.x * TILE;
-    const int cnt = min(TILE, n - s0);
-    for (int i = tid; i < NPARAM; i += GTHREADS) w[i] = theta[i];
-    for (int i = tid; i < TILE * D_IN; i += GTHREADS) {
-        const int r = i / D_IN, k = i % D_IN;
-        float v = 0.f;
-        if (r < cnt) {
-            const int sidx = idx ? idx[s0 + r] : s0 + r;
-            v = X[(size_t)sidx * D_IN + k];
-        }
-        xs[r][k] = v;
-    }
-    __syncthreads();
-    // z1 = W1 x + b1
-    for (int i = tid; i < TILE * H; i += GTHREADS) {
-        const int r = i / H, j = i % H;
-        float z = w[OFF_B1 + j];
-#pragma unroll
-        for (int k = 0; k < D_IN; ++k) z = fmaf(w[OFF_W1 + j * D_IN + k], xs[r][k], z);
-        z1[r][j] = z;
-    }
-    __syncthreads();
-    // z2 = W2 relu(z1) + b2
-    for (int i = tid; i < TILE * H; i += GTHREADS) {
-        const int r = i / H, j = i % H;
-        float z = w[OFF_B2 + j];
-        for (int k = 0; k < H; ++k) {
-            const float h = z1[r][k];
-            z = fmaf(w[OFF_W2 + j * H + k], h > 0.f ? h : 0.f, z);
-        }
-        z2[r][j] = z;
-    }
-    __syncthreads();
-    // y, residual, dL/dy = 2 (y - t) / n
-    if (tid < 32) {
-        float sq = 0.f, g = 0.f;
-        if (tid < cnt) {
-            float yv = w[OFF_B3];
-            for (int j = 0; j < H; ++j) {
-                const float h = z2[tid][j];
-                yv = fmaf(w[OFF_W3 + j], h > 0.f ? h : 0.f, yv);
+    constexpr int P = H + 4;                 // pitch of per-sample rows (16-byte aligned)
+    constexpr int Q = TILE >= 4 ? TILE / 4 : 1;   // samples per thread: r = tid / 64 + 4 q
+    __shared__ float w1[H * D_IN], b1[H], w2[H * (H + 1)], b2[H], w3[H];
+    __shared__ float b3, xs[TILE][D_IN], ts[TILE], dy[TILE], sq[TILE];
+    __shared__ __align__(16) float h1[TILE][P], h2[TILE][P], d2[TILE][P], d1[TILE][P];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int u = tid & (H - 1), r0 = tid >> 6;   // hidden unit and first sample of this thread
+    pdl_trigger();
+    pdl_wait();
+    for (int i = tid; i < H * D_IN; i += GTHREADS) w1[i] = theta[OFF_W1 + i];
+    for (int i = tid; i < H * H; i += GTHREADS) w2[(i >> 6) * (H + 1) + (i & (H - 1))] = theta[OFF_W2 + i];
+    if (tid < H) b1[tid] = theta[OFF_B1 + tid];
+    else if (tid < 2 * H) b2[tid - H] = theta[OFF_B2 + tid - H];
+    else if (tid < 3 * H) w3[tid - 2 * H] = theta[OFF_W3 + tid - 2 * H];
+    else if (tid == 3 * H) b3 = theta[OFF_B3];
+    // the thread's parameters: dW2[4 jb + a][4 kb + c], dW1[tid], dW1[tid + 256], one of the rest
+    const int jb = 4 * (tid >> 4), kb = 4 * (tid & 15);
+    float g2[4][4] = {}, g1[2] = {}, gb = 0.f, loss = 0.f;
+    const int tiles = (n + TILE - 1) / TILE;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int s0 = t * TILE, cnt = min(TILE, n - s0);
+        for (int i = tid; i < TILE * (D_IN + 1); i += GTHREADS) {
+            const int r = i / (D_IN + 1), k = i % (D_IN + 1);
+            float v = 0.f;
+            if (r < cnt) {
+                const int s = idx ? idx[s0 + r] : s0 + r;
+                v = k < D_IN ? X[(size_t)s * D_IN + k] : T[s];
             }
-            const int sidx = idx ? idx[s0 + tid] : s0 + tid;
-            const float r = yv - T[sidx];
-            sq = r * r;
-            g = 2.f * r / (float)n;
+            if (k < D_IN) xs[r][k] = v;
+            else ts[r] = v;
         }
-        if (tid < TILE) dy[tid] = g;
-        // tile sum of squared residuals (fixed order within the warp)
+        __syncthreads();
+        // h1 = relu(W1 x + b1)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        if (tid == 0) red[0] = sq;
+        for (int q = 0; q < Q; ++q) {
+            const int r = r0 + 4 * q;
+            if (r < TILE) {
+                float z = b1[u];
+#pragma unroll
+                for (int k = 0; k < D_IN; ++k) z = fmaf(w1[u * D_IN + k], xs[r][k], z);
+                h1[r][u] = z > 0.f ? z : 0.f;
+            }
+        }
+        __syncthreads();
+        // h2 = relu(W2 h1 + b2)
+        {
+            float z[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) z[q] = b2[u];
+            if (r0 < TILE) {
+#pragma unroll 4
+                for (int k = 0; k < H; k += 4) {
+                    const float* w = w2 + u * (H + 1) + k;
+                    const float a0 = w[0], a1 = w[1], a2 = w[2], a3 = w[3];
+#pragma unroll
+                    for (int q = 0; q < Q; ++q) {
+                        const float4 h = *reinterpret_cast<const float4*>(&h1[r0 + 4 * q][k]);
+                        z[q] = fmaf(a0, h.x, z[q]);
+                        z[q] = fmaf(a1, h.y, z[q]);
+                        z[q] = fmaf(a2, h.z, z[q]);
+                        z[q] = fmaf(a3, h.w, z[q]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < Q; ++q) h2[r0 + 4 * q][u] = z[q] > 0.f ? z[q] : 0.f;
+            }
+        }
+        __syncthreads();
+        // y, residual and dL/dy = 2 (y - t) / n: a warp per sample
+        for (int r = warp; r < TILE; r += GTHREADS / 32) {
+            float y = fmaf(w3[lane], h2[r][lane], w3[lane + 32] * h2[r][lane + 32]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+            const float e = r < cnt ? y + b3 - ts[r] : 0.f;
+            const float g = 2.f * e / (float)n;
+            if (lane == 0) {
+                dy[r] = g;
+                sq[r] = e * e;
+            }
+            // dL/dz2 = dy w3 [z2 > 0]
+            d2[r][lane] = h2[r][lane] > 0.f ? g * w3[lane] : 0.f;
+            d2[r][lane + 32] = h2[r][lane + 32] > 0.f ? g * w3[lane + 32] : 0.f;
+        }
+        __syncthreads();
+        // dL/dz1 = (W2^T dL/dz2) [z1 > 0]
+        if (r0 < TILE) {
+            float z[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) z[q] = 0.f;
+#pragma unroll 4
+            for (int j = 0; j < H; j += 4) {
+                const float* w = w2 + j * (H + 1) + u;
+                const float a0 = w[0], a1 = w[H + 1], a2 = w[2 * (H + 1)], a3 = w[3 * (H + 1)];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    const float4 d = *reinterpret_cast<const float4*>(&d2[r0 + 4 * q][j]);
+                    z[q] = fmaf(a0, d.x, z[q]);
+                    z[q] = fmaf(a1, d.y, z[q]);
+                    z[q] = fmaf(a2, d.z, z[q]);
+                    z[q] = fmaf(a3, d.w, z[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) d1[r0 + 4 * q][u] = h1[r0 + 4 * q][u] > 0.f ? z[q] : 0.f;
+        }
+        __syncthreads();
+        // parameter gradients, in sample order
+#pragma unroll
+        for (int r = 0; r < TILE; ++r) {
+            const float4 d = *reinterpret_cast<const float4*>(&d2[r][jb]);
+            const float4 h = *reinterpret_cast<const float4*>(&h1[r][kb]);
+            const float da[4] = {d.x, d.y, d.z, d.w}, hc[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) g2[a][c] = fmaf(da[a], hc[c], g2[a][c]);
+            g1[0] = fmaf(d1[r][tid / D_IN], xs[r][tid % D_IN], g1[0]);
+            if (tid + GTHREADS < H * D_IN)
+                g1[1] = fmaf(d1[r][(tid + GTHREADS) / D_IN], xs[r][(tid + GTHREADS) % D_IN], g1[1]);
+            if (tid < H) gb += d1[r][tid];
+            else if (tid < 2 * H) gb += d2[r][tid - H];
+            else if (tid < 3 * H) gb = fmaf(dy[r], h2[r][tid - 2 * H], gb);
+            else if (tid == 3 * H) gb += dy[r];
+            else if (tid == 3 * H + 1) loss += sq[r];
+        }
+        __syncthreads();   // the rows are reused by the next tile
     }
-    __syncthreads();
-    // dL/dz2 = dy * w3 * [z2 > 0]
-    for (int i = tid; i < TILE * H; i += GTHREADS) {
-        const int r = i / H, j = i % H;
-        d2[r][j] = z2[r][j] > 0.f ? dy[r] * w[OFF_W3 + j] : 0.f;
-    }
-    __syncthreads();
-    // dL/dz1 = (W2^T dL/dz2) * [z1 > 0]
-    for (int i = tid; i < TILE * H; i += GTHREADS) {
-        const int r = i / H, k = i % H;
-        float g = 0.f;
-        if (z1[r][k] > 0.f)
-            for (int j = 0; j < H; ++j) g = fmaf(w[OFF_W2 + j * H + k], d2[r][j], g);
-        d1[r][k] = g;
-    }
-    __syncthreads();
     float* out = partial + (size_t)blockIdx.x * (NPARAM + 1);
-    // parameter gradients summed over the tile's samples in sample order
-    for (int p = tid; p < NPARAM; p += GTHREADS) {
-        float g = 0.f;
-        if (p < OFF_B1) {
-            const int j = p / D_IN, k = p % D_IN;
-            for (int r = 0; r < TILE; ++r) g = fmaf(d1[r][j], xs[r][k], g);
-        } else if (p < OFF_W2) {
-            const int j = p - OFF_B1;
-            for (int r = 0; r < TILE; ++r) g += d1[r][j];
-        } else if (p < OFF_B2) {
-            const int j = (p - OFF_W2) / H, k = (p - OFF_W2) % H;
-            for (int r = 0; r < TILE; ++r) {
-                const float h = z1[r][k];
-                g = fmaf(d2[r][j], h > 0.f ? h : 0.f, g);
-            }
-        } else if (p < OFF_W3) {
-            const int j = p - OFF_B2;
-            for (int r = 0; r < TILE; ++r) g += d2[r][j];
-        } else if (p < OFF_B3) {
-            const int j = p - OFF_W3;
-            for (int r = 0; r < TILE; ++r) {
-                const float h = z2[r][j];
-                g = fmaf(dy[r], h > 0.f ? h : 0.f, g);
-            }
-        } else {
-            for (int r = 0; r < TILE; ++r) g += dy[r];
-        }
-        out[p] = g;
-    }
-    if (tid == 0) out[NPARAM] = red[0];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) out[OFF_W2 + (jb + a) * H + kb + c] = g2[a][c];
+    out[OFF_W1 + tid] = g1[0];
+    if (tid + GTHREADS < H * D_IN) out[OFF_W1 + tid + GTHREADS] = g1[1];
+    if (tid < H) out[OFF_B1 + tid] = gb;
+    else if (tid < 2 * H) out[OFF_B2 + tid - H] = gb;
+    else if (tid < 3 * H) out[OFF_W3 + tid - 2 * H] = gb;
+    else if (tid == 3 * H) out[OFF_B3] = gb;
+    else if (tid == 3 * H + 1) out[NPARAM] = loss;
 }
 
-// Sums the tile partials in tile order: grad[p] = sum_b partial[b][p]; the
-// last slot gives the loss (1/n) sum (y - t)^2.
-__global__ void __launch_bounds__(256) k_mlp_grad_reduce(int tiles, int n,
+// Sums the partials: thread (g, lane) adds partials g, g + 8, ... of parameter
+// 32 block + lane, the eight sums are added in order; the last slot gives the loss
+// (1/n) sum (y - t)^2.
+__global__ void __launch_bounds__(256) k_mlp_grad_reduce(int parts, int n,
                                                          const float* __restrict__ partial,
                                                          float* __restrict__ grad,
                                                          float* __restrict__ loss) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > NPARAM) return;
-    float g = 0.f;
-    for (int b = 0; b < tiles; ++b) g += partial[(size_t)b * (NPARAM + 1) + p];
-    if (p < NPARAM) grad[p] = g;
-    else loss[0] = g / (float)n;
+    __shared__ float s[8][32];
+    const int g = threadIdx.x >> 5, lane = threadIdx.x & 31, p = blockIdx.x * 32 + lane;
+    pdl_trigger();
+    pdl_wait();
+    float v = 0.f;
+    if (p <= NPARAM) {
+#pragma unroll 8
+        for (int b = g; b < parts; b += 8) v += partial[(size_t)b * (NPARAM + 1) + p];
+    }
+    s[g][lane] = v;
+    __syncthreads();
+    if (g == 0 && p <= NPARAM) {
+        for (int i = 1; i < 8; ++i) v += s[i][lane];
+        if (p < NPARAM) grad[p] = v;
+        else loss[0] = v / (float)n;
+    }
+}
+
+// The gradient's two launches over a scratch of grad_partials(n) partials.
+static pgk_status launch_grad(int n, const int* idx, const float* X, const float* t, const float* theta,
+                              float* grad, float* loss, float* partial, cudaStream_t s) {
+    const int parts = grad_partials(n);
+    void (*k)(int, const int*, const float*, const float*, const float*, float*) = k_mlp_grad_tile<16>;
+    switch (grad_tile(n)) {
+        case 2: k = k_mlp_grad_tile<2>; break;
+        case 4: k = k_mlp_grad_tile<4>; break;
+        case 8: k = k_mlp_grad_tile<8>; break;
+    }
+    PGK_CUDA_TRY(launch_pdl(k, (unsigned)parts, GTHREADS, 0, 1, s, n, idx, X, t, theta, partial),
+                 "MLP gradient launch");
+    PGK_CUDA_TRY(launch_pdl(k_mlp_grad_reduce, (unsigned)((NPARAM + 1 + 31) / 32), 256, 0, 1, s, parts, n,
+                            (const float*)partial, grad, loss),
+                 "MLP gradient launch");
+    return PGK_OK;
 }
 
 __global__ void k_adam(int count, float* __restrict__ theta, const float* __restrict__ grad,
                        float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2,
                        float eps, float bc1, float bc2) {
+    pdl_trigger();
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const float g = grad[i];
@@ -224,15 +303,11 @@ pgk_status pgk_mlp_loss_grad(int n, const int* idx, const float* X, const float*
         set_error("bad MLP gradient arguments (1 <= n <= 65536)");
         return PGK_ERR_INVALID_ARG;
     }
-    const int tiles = (n + TILE - 1) / TILE;
     pgk_status st;
-    float* partial = (float*)workspace(WS_PARTIAL, sizeof(float) * (size_t)tiles * (NPARAM + 1), &st);
+    float* partial =
+        (float*)workspace(WS_PARTIAL, sizeof(float) * (size_t)grad_partials(n) * (NPARAM + 1), &st);
     if (!partial) return st;
-    cudaStream_t s = (cudaStream_t)stream;
-    k_mlp_grad_tile<<<tiles, GTHREADS, 0, s>>>(n, idx, X, t, theta, partial);
-    k_mlp_grad_reduce<<<(NPARAM + 1 + 255) / 256, 256, 0, s>>>(tiles, n, partial, grad, loss);
-    PGK_CUDA_TRY(cudaGetLastError(), "MLP gradient launch");
-    return PGK_OK;
+    return launch_grad(n, idx, X, t, theta, grad, loss, partial, (cudaStream_t)stream);
 }
 
 pgk_status pgk_mlp_adam(int count, float* theta, const float* grad, float* m, float* v, int step,
@@ -243,9 +318,9 @@ pgk_status pgk_mlp_adam(int count, float* theta, const float* grad, float* m, fl
     }
     const float bc1 = (float)(1.0 - pow((double)beta1, (double)step));
     const float bc2 = (float)(1.0 - pow((double)beta2, (double)step));
-    k_adam<<<(count + 255) / 256, 256, 0, (cudaStream_t)stream>>>(count, theta, grad, m, v, lr, beta1,
-                                                                  beta2, eps, bc1, bc2);
-    PGK_CUDA_TRY(cudaGetLastError(), "Adam launch");
+    PGK_CUDA_TRY(launch_pdl(k_adam, (unsigned)((count + 255) / 256), 256, 0, 1, (cudaStream_t)stream, count, theta,
+                            grad, m, v, lr, beta1, beta2, eps, bc1, bc2),
+                 "Adam launch");
     return PGK_OK;
 }
 
@@ -259,7 +334,7 @@ pgk_status pgk_mlp_adam(int count, float* theta, const float* grad, float* m, fl
 // in a file-scope device array sized for PGK_MLP_NOALLOC_MAX_SAMPLES samples.
 // Every GPU that loads the library holds this array until the process exits.
 namespace pgk {
-static constexpr int NOALLOC_TILES = PGK_MLP_NOALLOC_MAX_SAMPLES / TILE;
+static constexpr int NOALLOC_TILES = PGK_MLP_NOALLOC_MAX_SAMPLES / 16;
 static __device__ __align__(256) float g_mlp_noalloc_partial[NOALLOC_TILES * (NPARAM + 1)];
 
 static std::mutex g_noalloc_mu;
@@ -310,10 +385,5 @@ extern "C" pgk_status pgk_mlp_loss_grad_noalloc(int n, const int* idx, const flo
     float* partial = nullptr;
     pgk_status st = noalloc_scratch(&partial);
     if (st != PGK_OK) return st;
-    const int tiles = (n + TILE - 1) / TILE;
-    cudaStream_t s = (cudaStream_t)stream;
-    k_mlp_grad_tile<<<tiles, GTHREADS, 0, s>>>(n, idx, X, t, theta, partial);
-    k_mlp_grad_reduce<<<(NPARAM + 1 + 255) / 256, 256, 0, s>>>(tiles, n, partial, grad, loss);
-    PGK_CUDA_TRY(cudaGetLastError(), "MLP gradient launch");
-    return PGK_OK;
+    return launch_grad(n, idx, X, t, theta, grad, loss, partial, (cudaStream_t)stream);
 }

@@ -142,3 +142,20 @@ def test_planned_tensor_core_program(dev, form, M, N, K, pad, beta):
     want = A.double() @ B.double() + (C0.double() if beta else 0)
     assert torch.equal(C[:, :N].double(), want)
     assert torch.isnan(C[:, N:]).all()
+
+
+@pytest.mark.parametrize("n", [2, 3, 255, 257, 511, 513, 1023, 1025, 2047, 4865])
+def test_cost_model_gradient_at_tile_edges(dev, n):
+    """Sizes at which the tile of a gradient block changes (2, 4, 8, 16 samples), with a
+    ragged last tile, and more tiles than blocks; the bar of the gradient tests."""
+    from oracle import mlp
+    rng = np.random.default_rng(n)
+    X, t = rng.standard_normal((n, 7)).astype(np.float32), rng.standard_normal(n).astype(np.float32)
+    th = inputs.he_uniform_mlp(n) + rng.normal(0, 0.05, pgk.MLP_PARAMS).astype(np.float32)
+    g, loss = torch.full((pgk.MLP_PARAMS,), float("nan"), device=dev), torch.zeros(1, device=dev)
+    pgk.mlp_loss_grad(*(torch.from_numpy(a).to(dev) for a in (X, t, th)), g, loss)
+    L, want = mlp.loss_and_grad(th.astype(np.float64), X.astype(np.float64), t.astype(np.float64))
+    assert abs(loss.item() - L) <= 1e-5 * abs(L)
+    got = mlp.unpack(g.cpu().numpy().astype(np.float64))
+    for name, b in mlp.unpack(want).items():
+        assert np.linalg.norm(got[name] - b) <= 1e-4 * max(np.linalg.norm(b), 1e-12), name
