@@ -335,8 +335,10 @@ PGK_API pgk_status pgk_select_case_jacobi(const pgk_machine* machine, const int*
 /* `steps` time steps of 1D Jacobi on the int32 device array a[2n]: step t
  * writes one half from the three-point average of the other (t odd: a[p+1] =
  * (a[n+p] + a[n+p+1] + a[n+p+2]) / 3, else a[n+p+1] = (a[p] + a[p+1] + a[p+2])
- * / 3) for every p in [0, n-2), C integer division.  One launch per step.
- * prog NULL = (B, s) = (128, 2), the paper's best.  n >= 3.
+ * / 3) for every p in [0, n-2), C integer division.  One launch per step;
+ * prog NULL = all steps in one cooperative launch where its blocks can hold the
+ * array (about 3.8 million points) and the stream is not being captured, else
+ * (B, s) = (128, 2), the paper's best, or (128, 8) from 2^20 points.  n >= 3.
  * Errors: INVALID_ARG, INFEASIBLE, UNSUPPORTED, CUDA. */
 PGK_API pgk_status pgk_jacobi(int n, int steps, int32_t* a, const pgk_params* prog, void* stream);
 

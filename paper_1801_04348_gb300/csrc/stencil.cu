@@ -20,6 +20,7 @@
 //   (3b,4a)  the same with s = 1,
 //   (3b,4b)  no shared memory.
 // One launch per time step (the halves swap roles between steps).
+#include <cooperative_groups.h>
 #include <string.h>
 
 #include <algorithm>
@@ -216,6 +217,93 @@ __global__ void k_jacobi_direct(int n, int odd, int32_t* a) {
     const int32_t* src = odd ? a + n : a;
     int32_t* dst = odd ? a : a + n;
     if (pp < n - 2) dst[pp + 1] = (src[pp] + src[pp + 1] + src[pp + 2]) / 3;
+}
+
+// Several time steps in one cooperative launch, for calls without parameters whose array the
+// blocks can hold: block b keeps interior points [1 + b R, 1 + (b + 1) R) in shared memory
+// with a halo of up to JSTEPS points a side, and recomputes the halo instead of exchanging
+// it.  A group of up to JSTEPS steps reads its window from the first half, waits until every
+// block has read (the group overwrites both halves), takes the steps, and writes the results
+// of the last two, which are what the halves then hold.  The end points of each half never
+// change.  A launch per step pays 4.1 us each, and at the paper's length 2^15 + 2 the work
+// of a step is far below that: 4 steps take 6.1 us instead of 16.4, at 2^20 + 2 points 10.4
+// instead of 24.7 (20.4 with granularity 8).
+static constexpr int JSTEPS = 8;   // even: every group starts from the first half
+static constexpr int JTHREADS = 512;
+
+__global__ void __launch_bounds__(JTHREADS, 2) k_jacobi_steps(int n, int steps, int R, int32_t* a) {
+    extern __shared__ int32_t buf_j[];   // two windows of R + 2 JSTEPS points
+    const int lo = 1 + (int)min((long long)blockIdx.x * R, (long long)(n - 2));
+    const int hi = lo + min(R, n - 1 - lo);   // own points [lo, hi)
+    int32_t* cur = buf_j;
+    int32_t* nxt = buf_j + R + 2 * JSTEPS;
+    for (int t0 = 0; t0 < steps; t0 += JSTEPS) {
+        const int s = min(JSTEPS, steps - t0);
+        const int w0 = max(0, lo - s), w1 = min(n, hi + s);   // window [w0, w1)
+        for (int i = w0 + (int)threadIdx.x; i < w1; i += JTHREADS) cur[i - w0] = a[i];
+        // end points of the second half (those of the first lie in the windows that need them)
+        const int32_t b0 = a[n], b1 = a[2 * (size_t)n - 1], c0 = a[0], c1 = a[n - 1];
+        if (s > 1) cooperative_groups::this_grid().sync();
+        else __syncthreads();
+        for (int k = 1; k <= s; ++k) {
+            const bool odd = k & 1;   // step t0 + k - 1 is even and writes the second half
+            int32_t* half = odd ? a + n : a;
+            const int p0 = max(0, lo - (s - k)), p1 = min(n, hi + (s - k));
+            for (int i = p0 + (int)threadIdx.x; i < p1; i += JTHREADS) {
+                const int j = i - w0;
+                int32_t v;
+                if (i == 0) v = odd ? b0 : c0;
+                else if (i == n - 1) v = odd ? b1 : c1;
+                else v = (cur[j - 1] + cur[j] + cur[j + 1]) / 3;
+                nxt[j] = v;
+                if (k >= s - 1 && i >= lo && i < hi) half[i] = v;
+            }
+            __syncthreads();
+            int32_t* const t = cur;
+            cur = nxt;
+            nxt = t;
+        }
+        if (t0 + JSTEPS < steps) cooperative_groups::this_grid().sync();
+    }
+}
+
+// Launches k_jacobi_steps; false if it does not apply (one step, an array too long for the
+// blocks' shared memory, a stream being captured, blocks that cannot all be resident): the
+// caller then launches every step.
+static bool launch_jacobi_steps(int n, int steps, int32_t* a, cudaStream_t st, cudaError_t* err) {
+    pgk_machine m;
+    if (steps < 2 || current_machine(&m, NULL) != PGK_OK) return false;
+    // at least JTHREADS points per block, two blocks per SM, their windows within 100 KB
+    const int blocks = (int)std::min<long long>(((long long)n - 2 + JTHREADS - 1) / JTHREADS, 2LL * m.sm_count);
+    const long long R = ((long long)n - 2 + blocks - 1) / blocks;
+    const long long smem = 8 * (R + 2 * JSTEPS);
+    if (smem > 100 * 1024 || 2 * (smem + 1024) > 227 * 1024) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    static SmemLimit limit;
+    if (allow_smem(limit, (const void*)k_jacobi_steps, 100 * 1024) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+    cfg.blockDim = dim3(JTHREADS, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    *err = cudaLaunchKernelEx(&cfg, k_jacobi_steps, n, steps, (int)R, a);
+    if (*err == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
 }
 
 // ----------------------------------------------------------- variant tables
@@ -512,7 +600,14 @@ pgk_status pgk_jacobi(int n, int steps, int32_t* a, const pgk_params* prog, void
     pgk_machine m;
     pgk_status st = current_machine(&m, NULL);
     if (st != PGK_OK) return st;
-    pgk_params p = {128, 1, 2, 1, 0};  // the paper's best: block 128, granularity 2 (Table Jacobi)
+    // without parameters: the steps of one launch where the blocks can hold the array, else a
+    // launch per step at the paper's best block (128, granularity 2: Table Jacobi), with
+    // granularity 8 from 2^20 points on, where HBM and not the launch bounds a step
+    // (4 steps at 2^26 points: 393 us, 788 with granularity 2)
+    cudaError_t e = cudaSuccess;
+    if (!prog && launch_jacobi_steps(n, steps, a, (cudaStream_t)stream, &e))
+        return e == cudaSuccess ? PGK_OK : cuda_fail(e, "Jacobi launch");
+    pgk_params p = {128, 1, n >= (1 << 20) ? 8 : 2, 1, 0};
     if (prog) p = *prog;
     pgk_case c;
     if ((st = stencil_case(KIND_JACOBI, &m, NULL, &p, &c)) != PGK_OK) return st;

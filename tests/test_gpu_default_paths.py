@@ -159,3 +159,30 @@ def test_cost_model_gradient_at_tile_edges(dev, n):
     got = mlp.unpack(g.cpu().numpy().astype(np.float64))
     for name, b in mlp.unpack(want).items():
         assert np.linalg.norm(got[name] - b) <= 1e-4 * max(np.linalg.norm(b), 1e-12), name
+
+
+@pytest.mark.parametrize("n", [3, 4, 6, 100, 513, 514, 515, 1026, 32770, 200001, 4200000])
+@pytest.mark.parametrize("steps", [0, 1, 2, 3, 8, 9, 17])
+def test_jacobi_without_parameters(dev, n, steps):
+    """Steps fused in one cooperative launch (groups of eight, blocks of 512 points and more,
+    the last one ragged or empty) and, beyond what the blocks hold, one launch per step:
+    exact, end points and both halves included."""
+    from oracle import stencil
+    a = np.random.default_rng(n + steps).integers(-10 ** 9 // 3, 10 ** 9 // 3, 2 * n).astype(np.int32)
+    ad = torch.from_numpy(a).to(dev)
+    pgk.jacobi(ad, n, steps)
+    assert np.array_equal(ad.cpu().numpy(), stencil.jacobi(a, n, steps))
+
+
+def test_jacobi_without_parameters_in_a_graph(dev):
+    """A captured call takes the launch per step."""
+    from oracle import stencil
+    n, steps = 1000, 5
+    a = np.random.default_rng(1).integers(-1000, 1000, 2 * n).astype(np.int32)
+    ad = torch.from_numpy(a).to(dev)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        pgk.jacobi(ad, n, steps)
+    ad.copy_(torch.from_numpy(a))
+    g.replay()
+    assert np.array_equal(ad.cpu().numpy(), stencil.jacobi(a, n, steps))
