@@ -75,6 +75,13 @@ void* workspace(int slot, size_t bytes, pgk_status* st) {
     return ptr;
 }
 
+bool workspace_ready(int slot, size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return false;
+    std::lock_guard<std::mutex> lk(g_ws_mu);
+    return g_ws_ptr[dev][slot] && g_ws_size[dev][slot] >= bytes;
+}
+
 unsigned int* device_error_word(pgk_status* st) {
     *st = PGK_OK;
     int dev = 0;

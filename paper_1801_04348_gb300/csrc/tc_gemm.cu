@@ -18,8 +18,9 @@
 // The fused-conversion programs (128 x 64 tiles, N <= 64) add eight converter
 // warps after the epilogue warps: the producer loads A in FP32 into a ring of its
 // own and only B^T into the stages; the converters write A's BF16 tiles (hi, and
-// lo for split) into the stages.  Their work units may be K slices of a tile,
-// whose partial products k_slice_reduce sums in slice order.
+// lo for split) into tensor memory.  Their work units may be K slices of a tile, whose
+// partial products k_slice_reduce sums in slice order, or contiguous ranges of the K
+// blocks of all tiles, whose pieces k_stream_reduce sums.
 // A product with few tiles may run each as a cluster of CTAs, one K slice per CTA (KSPLIT):
 // the partial tiles meet in shared memory and every CTA sums a slab of rows over its peers.
 // Every wait is bounded (globaltimer); on timeout the CTA sets the device
@@ -66,8 +67,11 @@ struct TcCfg {
     static constexpr bool PAIR = PAIR_;
     // Fused conversion (FSTAGES > 0): A arrives in FP32 through an FSTAGES-deep ring
     // (per K block two TMA boxes of 128 rows x 32 FP32, 128B-swizzled) and converter
-    // warps write its BF16 tiles (hi, and lo for split) into the stage ring, so A is
+    // warps write its BF16 tiles (hi, and lo for split) into tensor memory, where the MMA
+    // takes its A operand from (one lane per row, two K columns per 32-bit word), so A is
     // read from memory once; only B^T (prepared, BF16) travels by TMA into the stages.
+    // Bound by HBM latency: the ring holds what is in flight, and A in tensor memory instead
+    // of the stages leaves room for five slots (160 KB) instead of two (split) or three.
     static constexpr int FSTAGES = FSTAGES_;
     static constexpr bool FUSED = FSTAGES > 0;
     static constexpr int BM = 128;                          // rows of A staged (and accumulated) per CTA
@@ -81,7 +85,7 @@ struct TcCfg {
     static constexpr int B_BYTES = BNL * 128;
     static constexpr int NOPS = MODE == MODE_SPLIT ? 2 : 1; // hi/lo pairs per stage
     static constexpr int PASSES = MODE == MODE_SPLIT3 ? 3 : 1;  // stages per K block
-    static constexpr int STAGE_BYTES = NOPS * (A_BYTES + B_BYTES);
+    static constexpr int STAGE_BYTES = NOPS * ((FUSED ? 0 : A_BYTES) + B_BYTES);
     // K blocks accumulated in tensor memory before the epilogue folds the chunk
     // into FP32 registers (0 = whole K in tensor memory).  FP8: every 128-deep
     // chunk carries its own scales.  Split: 512-deep chunks bound the growth
@@ -96,12 +100,27 @@ struct TcCfg {
     // MMA's completion to the reuse of its accumulator
     static constexpr bool POLL = MODE == MODE_FP8;
     static constexpr int CONV_WARPS = FUSED ? 8 : 0;        // warps after the epilogue warps
+    // the converters work in two groups of four warps on alternate K blocks: a block's
+    // chain (wait, shared loads, conversions, tensor-memory stores, arrival) is latency, and
+    // two blocks are then in it
+    static constexpr int CONV_GROUP = CONV_WARPS / 2;
     static constexpr int THREADS = 64 + 32 * (EPI_WARPS + CONV_WARPS);
     static constexpr int F_BYTES = FUSED ? 2 * BM * 128 : 0;  // one FP32 K block of A (two boxes)
     // tensor-memory accumulators in flight: FP8 with 128-wide tiles keeps four
     // chunk accumulators so the MMA can run three chunks ahead of the epilogue
     static constexpr int ACC_BUFS = (MODE == MODE_FP8 && BN == 128) ? 4 : 2;
-    static constexpr int TMEM_COLS = ACC_BUFS * BN;
+    // fused: each stage's A (32 columns per 64-deep BF16 tile) after the accumulators
+    // Fused split launches over K ranges issue two MMAs per K step instead of three (DUAL): a
+    // 128 x 64 MMA takes the tensor pipe as long as a 128 x 128 one (128 cycles measured), so
+    // the twelve of a K block took 1560 cycles and bounded the program.  B hi and lo lie one
+    // after the other in the stage, and A hi meets both in one 128-wide MMA, whose halves
+    // accumulate hi*hi and the cross terms apart.  Programs of whole slices keep the three
+    // (and the sums of the two-pass programs, bit for bit).
+    static constexpr bool DUAL = FSTAGES_ > 0 && MODE == MODE_SPLIT;
+    static constexpr int ACC_COLS = DUAL ? 2 * BN : BN;   // columns of an accumulator (pair)
+    static constexpr int TMEM_A = ACC_BUFS * ACC_COLS, TMEM_A_STAGE = NOPS * 32;
+    static constexpr int TMEM_COLS = FUSED ? 512 : ACC_BUFS * BN;
+    static_assert(!FUSED || TMEM_A + STAGES * TMEM_A_STAGE <= 512, "A stages fit tensor memory");
     // epilogue staging: one 32 x 32 FP32 block per epilogue warp after the stage ring
     static constexpr int XPOSE_BYTES = EPI_WARPS * 32 * 32 * 4;
     static constexpr int SMEM_RAW = STAGES * STAGE_BYTES + FSTAGES * F_BYTES + XPOSE_BYTES + 1024;
@@ -239,6 +258,15 @@ __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint
         "l"(a), "l"(b), "r"(idesc), "r"(accum));
 }
 
+// The same with A in tensor memory (a: its first column).
+__device__ __forceinline__ void mma_f16_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc,
+                                           uint32_t accum) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+        "r"(a), "l"(b), "r"(idesc), "r"(accum));
+}
+
 __device__ __forceinline__ void mma_f8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                        uint32_t accum) {
     asm volatile(
@@ -267,6 +295,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
           "=r"(r[31])
         : "r"(taddr));
+}
+
+// 16 registers per thread -> 32 TMEM lanes x 16 consecutive 32-bit columns.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+        "%11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // Paired FP32 arithmetic for the chunk fold: two IEEE fused multiply-adds
@@ -394,7 +435,16 @@ struct TcParams {
     // launches: slice s is CTA s of the tile's cluster
     int kslices, kper;
     float* part;
+    // fused-conversion programs over K ranges: the K blocks of all tiles, in order, are cut
+    // into `stream` contiguous ranges, one per CTA (0: off).  A tile that one range covers
+    // goes to C; the piece that a range holds of its first tile goes to slot 2 CTA of part,
+    // of a later one to slot 2 CTA + 1 (128 x N floats each), and k_stream_reduce adds them
+    int stream;
 };
+
+// First unit of range g of G over U units, and the range that holds unit x.
+__host__ __device__ inline long long range_begin(int g, int G, long long U) { return g * U / G; }
+__host__ __device__ inline int range_of(long long x, int G, long long U) { return (int)(((x + 1) * G - 1) / U); }
 
 // Tensor maps of one launch: A and B^T (hi, and lo for the split forms), and B^T
 // with half-height boxes for the column halves of tail-balanced tiles.
@@ -468,18 +518,24 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
     const int tail = TAIL ? p.tail : 0;
     // work units: every tile, the last `tail` of them twice (one per column half)
     const int ksl = ((Cfg::FUSED || KSPLIT) && p.kslices > 1) ? p.kslices : 1;
-    const int ntiles = GROUPED ? p.ntiles_g : (nfull + tail) * ksl;
     const int nkb = (p.K + Cfg::BK - 1) / Cfg::BK;
+    auto stream_pieces = [&] {   // tiles that this CTA's K range touches
+        const long long U = (long long)nfull * nkb;
+        return (int)((range_begin(blockIdx.x + 1, p.stream, U) - 1) / nkb -
+                     range_begin(blockIdx.x, p.stream, U) / nkb) + 1;
+    };
+    const int ntiles = GROUPED ? p.ntiles_g
+                       : Cfg::FUSED && p.stream > 0 ? stream_pieces() : (nfull + tail) * ksl;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::STAGES; ++s) {
-            // fused: the producer's B^T copies and one arrival per converter warp
-            mbar_init(&full_bar[s], 1 + Cfg::CONV_WARPS);
+            // fused: the producer's B^T copies and one arrival per converter warp of a group
+            mbar_init(&full_bar[s], 1 + Cfg::CONV_GROUP);
             mbar_init(&empty_bar[s], 1);
         }
         for (int s = 0; s < Cfg::FSTAGES; ++s) {
             mbar_init(&ffull_bar[s], 1);
-            mbar_init(&fempty_bar[s], Cfg::CONV_WARPS);
+            mbar_init(&fempty_bar[s], Cfg::CONV_GROUP);
         }
         for (int b = 0; b < Cfg::ACC_BUFS; ++b) {
             mbar_init(&accf_bar[b], 1);
@@ -536,12 +592,15 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
         tm = first + r % gm;
         tn = r / gm;
     };
+    // the CTA's first work unit and its stride: tiles of the grid, or pieces of its K range
+    auto first_unit = [&] { return Cfg::FUSED && p.stream > 0 ? 0 : tile_first<PAIR>(); };
+    auto unit_stride = [&] { return Cfg::FUSED && p.stream > 0 ? 1u : tile_stride<PAIR>(); };
     // everything a warp needs about tile t: its position, its problem's sizes and
     // output, and where its operands start in the packed workspaces (grouped)
     struct TileInfo {
         int tm, tn, M, N, nkb, rowA, rowB, ldc;
         int half;   // -1: the whole tile; 0 or 1: its first or second BN/2 columns
-        int kb0;    // first K block (a K slice of a fused-conversion program), else 0
+        int kb0;    // first K block (a K slice or range), else 0
         int beta;
         float* C;
     };
@@ -566,6 +625,8 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             int tt = t;
             ti.half = -1;
             int sl = 0;
+            const bool stream = Cfg::FUSED && p.stream > 0;
+            if (stream) tt = (int)(range_begin(blockIdx.x, p.stream, (long long)nfull * nkb) / nkb) + t;
             if ((Cfg::FUSED || KSPLIT) && ksl > 1) {
                 sl = t % ksl;
                 tt = t / ksl;
@@ -589,6 +650,22 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                 ti.kb0 = sl * p.kper;
                 ti.nkb = min(nkb - ti.kb0, p.kper);
             }
+            if (stream) {
+                // piece t of this CTA's range: tile tt from its begin (the first piece) to
+                // its end (the last one)
+                const long long U = (long long)nfull * nkb, base = (long long)tt * nkb;
+                const long long u0 = range_begin(blockIdx.x, p.stream, U);
+                const long long u1 = range_begin(blockIdx.x + 1, p.stream, U);
+                ti.kb0 = t == 0 ? (int)(u0 - base) : 0;
+                const int end = (int)min((long long)nkb, u1 - base);
+                if (ti.kb0 > 0 || end < nkb) {
+                    // (rows of the piece are addressed by their rows in C)
+                    ti.C = p.part + ((long long)(2 * blockIdx.x + (t > 0)) - ti.tm) * Cfg::BM * p.N;
+                    ti.ldc = p.N;
+                    ti.beta = 0;
+                }
+                ti.nkb = end - ti.kb0;
+            }
             if (Cfg::FUSED && ksl > 1) {
                 ti.kb0 = sl * p.kper;
                 ti.nkb = min(nkb - ti.kb0, p.kper);
@@ -610,7 +687,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             uint32_t phase = 0, fphase = 0;
             uint32_t issued = 0, parity = 0, fissued = 0, fparity = 0;
             bool ok = true;
-            for (int t = tile_first<PAIR>(); t < ntiles && ok; t += tile_stride<PAIR>()) {
+            for (int t = first_unit(); t < ntiles && ok; t += unit_stride()) {
                 const TileInfo ti = tile_info(t);
                 const int ya = ti.tm * Cfg::TM;
                 const int yb = ti.tn * Cfg::BN;
@@ -638,9 +715,8 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                     }
                     uint8_t* st = tiles + (size_t)stage * Cfg::STAGE_BYTES;
                     mbar_arrive_expect_tx(&full_bar[stage], (uint32_t)(Cfg::NOPS * Cfg::B_BYTES));
-                    tma_load_2d(st + Cfg::A_BYTES, &tm.b, &full_bar[stage], x, yb);
-                    if (Cfg::MODE == MODE_SPLIT)
-                        tma_load_2d(st + 2 * Cfg::A_BYTES + Cfg::B_BYTES, &tm.b2, &full_bar[stage], x, yb);
+                    tma_load_2d(st, &tm.b, &full_bar[stage], x, yb);
+                    if (Cfg::MODE == MODE_SPLIT) tma_load_2d(st + Cfg::B_BYTES, &tm.b2, &full_bar[stage], x, yb);
                     issued |= 1u << stage;
                     parity = (parity & ~(1u << stage)) | (phase << stage);
                     if (++stage == Cfg::STAGES) {
@@ -682,7 +758,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             uint32_t phase = 0;
             uint32_t issued_mask = 0, last_parity = 0;
             bool ok = true;
-            for (int t = tile_first<PAIR>(); t < ntiles && ok; t += tile_stride<PAIR>()) {
+            for (int t = first_unit(); t < ntiles && ok; t += unit_stride()) {
                 const TileInfo ti = tile_info(t);
                 const bool hf = ti.half >= 0;
                 // B^T rows staged by this CTA: BNL, or BNL/2 for a column half
@@ -773,7 +849,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
             uint32_t acc_phase = 0;
             bool ok = true;
             bool issued_any = false;
-            for (int t = tile_first<PAIR>(); t < ntiles && ok; t += tile_stride<PAIR>()) {
+            for (int t = first_unit(); t < ntiles && ok; t += unit_stride()) {
                 const TileInfo ti = tile_info(t);
                 const int tnkb = ti.nkb;
                 const uint32_t idesc = ti.half >= 0 ? idesc_half : idesc_full;
@@ -802,16 +878,41 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t d = tmem_base + (uint32_t)(acc * Cfg::BN);
+                        const uint32_t d = tmem_base + (uint32_t)(acc * Cfg::ACC_COLS);
                         const uint32_t sa = smem_u32(tiles + (size_t)stage * Cfg::STAGE_BYTES);
                         const uint32_t sb = sa + Cfg::A_BYTES;
+                        if (Cfg::DUAL && p.stream > 0) {
+                            // columns 0 .. BN - 1: hi*hi; BN .. 2 BN - 1: hi*lo and lo*hi
+                            const uint32_t idesc_two = idesc_bf16(Cfg::TM, 2 * Cfg::BN);
+#pragma unroll
+                            for (int ks = 0; ks < Cfg::NKSUB; ++ks) {
+                                const uint32_t ta = tmem_base + (uint32_t)(Cfg::TMEM_A + stage * Cfg::TMEM_A_STAGE +
+                                                                           ks * 8);
+                                const uint64_t fb = sdesc_k128(sa + ks * 32u);
+                                mma_f16_ta(d, ta, fb, idesc_two, (kin > 0 || ks > 0) ? 1u : 0u);
+                                mma_f16_ta(d + Cfg::BN, ta + 32u, fb, idesc, 1u);
+                            }
+                        } else
 #pragma unroll
                         for (int ks = 0; ks < Cfg::NKSUB; ++ks) {
                             const uint32_t koff = (uint32_t)ks * 32u;  // 32 bytes of K per MMA
                             const uint64_t da = sdesc_k128(sa + koff);
                             const uint64_t db = sdesc_k128(sb + koff);
                             const uint32_t accum = (kin > 0 || v > 0 || ks > 0) ? 1u : 0u;
-                            if (Cfg::MODE == MODE_FP8) {
+                            if (Cfg::FUSED) {
+                                // A hi (and lo) in tensor memory, B hi (and lo) in the stage
+                                const uint32_t ta = tmem_base + (uint32_t)(Cfg::TMEM_A + stage * Cfg::TMEM_A_STAGE +
+                                                                           ks * 8);
+                                const uint64_t fb = sdesc_k128(sa + koff);
+                                if (Cfg::MODE == MODE_SPLIT) {
+                                    const uint64_t fb2 = sdesc_k128(sa + Cfg::B_BYTES + koff);
+                                    mma_f16_ta(d, ta + 32u, fb, idesc, accum);
+                                    mma_f16_ta(d, ta, fb2, idesc, 1u);
+                                    mma_f16_ta(d, ta, fb, idesc, 1u);
+                                } else {
+                                    mma_f16_ta(d, ta, fb, idesc, accum);
+                                }
+                            } else if (Cfg::MODE == MODE_FP8) {
                                 mma_f8(d, da, db, idesc, accum);
                             } else if (PAIR && (Cfg::MODE == MODE_BF16 || Cfg::MODE == MODE_SPLIT3)) {
                                 mma_f16_pair(d, da, db, idesc, accum);
@@ -888,75 +989,79 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
         __syncwarp();
     } else if (Cfg::FUSED && warp >= 2 + Cfg::EPI_WARPS) {
         // ------------------------------------------------------- converters
-        // thread (r, h): row r of the 128-row block, FP32 box h (K columns 32h ..
-        // 32h + 31 of the 64-deep block).  The 16-byte chunk i of a 128-byte row
-        // sits at chunk i ^ (r mod 8) (128-byte swizzle) in the FP32 boxes and in
-        // the BF16 operand tiles alike, so eight consecutive rows of a quarter warp
-        // touch eight different chunks: no bank conflicts either way.
-        const int ct = (int)threadIdx.x - 32 * (2 + Cfg::EPI_WARPS);
-        const int r = ct & 127, h = ct >> 7;
+        // thread: row r of the 128-row block, FP32 box h (K columns 32h .. 32h + 31 of the
+        // 64-deep block) for h = 0, 1.  The 16-byte chunk i of a 128-byte row
+        // sits at chunk i ^ (r mod 8) (128-byte swizzle) in the FP32 boxes, so eight
+        // consecutive rows of a quarter warp touch eight different chunks: no bank
+        // conflicts.  A warp reaches the tensor-memory lanes 32 (warp mod 4) .. + 31
+        // only, which fixes its rows; the row's 32 values are 16 words there.
+        const int tq = warp & 3, r = tq * 32 + lane;
+        const unsigned group = (unsigned)(warp - (2 + Cfg::EPI_WARPS)) / Cfg::CONV_GROUP;
         const int rx = r & 7;
+        unsigned turn = 0;   // K blocks so far: the group takes every second one
         int stage = 0, fs = 0;
         uint32_t phase = 0, fphase = 0;
         bool ok = true;
-        for (int t = tile_first<PAIR>(); t < ntiles && ok; t += tile_stride<PAIR>()) {
+        for (int t = first_unit(); t < ntiles && ok; t += unit_stride()) {
             const TileInfo ti = tile_info(t);
             for (int kb = 0; kb < ti.nkb; ++kb) {
-                int w = 1;
-                if (lane == 0)
-                    w = (mbar_wait<Cfg::POLL>(&ffull_bar[fs], fphase, abort_flag, p.err,
-                                              ERR_TIMEOUT_PRODUCER) &&
-                         mbar_wait<Cfg::POLL>(&empty_bar[stage], phase ^ 1u, abort_flag, p.err,
-                                              ERR_TIMEOUT_PRODUCER)) ? 1 : 0;
-                w = __shfl_sync(0xffffffffu, w, 0);
-                if (!w) {
-                    ok = false;
-                    break;
-                }
-                // every lane observes both completed phases (lane 0 already has)
-                while (!mbar_test_wait(&ffull_bar[fs], fphase)) {
-                }
-                while (!mbar_test_wait(&empty_bar[stage], phase ^ 1u)) {
-                }
-                const uint8_t* src = fring + (size_t)fs * Cfg::F_BYTES + h * (Cfg::F_BYTES / 2) + r * 128;
-                float4 v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    v[i] = *reinterpret_cast<const float4*>(src + ((i ^ rx) << 4));
-                // the FP32 slot is free once every lane of every converter warp has read it
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&fempty_bar[fs]);
-                uint8_t* dhi = tiles + (size_t)stage * Cfg::STAGE_BYTES + r * 128;
-                uint8_t* dlo = dhi + Cfg::A_BYTES + Cfg::B_BYTES;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    // K columns 32h + 8i .. 32h + 8i + 7 -> 16-byte chunk 4h + i of the BF16 row
-                    const float x[8] = {v[2 * i].x, v[2 * i].y, v[2 * i].z, v[2 * i].w,
-                                        v[2 * i + 1].x, v[2 * i + 1].y, v[2 * i + 1].z, v[2 * i + 1].w};
-                    // a pair of columns per 32-bit word, lower column in the lower half:
-                    // hi = bf16(x) and lo = bf16(x - hi), both rounded to nearest even
-                    // (x - hi is exact in FP32)
-                    uint32_t hw[4], lw[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const __nv_bfloat162 hp = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-                        hw[j] = *reinterpret_cast<const uint32_t*>(&hp);
-                        if (Cfg::MODE == MODE_SPLIT) {
-                            const float2 hf = __bfloat1622float2(hp);
-                            const __nv_bfloat162 lp =
-                                __floats2bfloat162_rn(x[2 * j] - hf.x, x[2 * j + 1] - hf.y);
-                            lw[j] = *reinterpret_cast<const uint32_t*>(&lp);
-                        }
+                if ((turn++ & 1u) == group) {
+                    int w = 1;
+                    if (lane == 0)
+                        w = (mbar_wait<Cfg::POLL>(&ffull_bar[fs], fphase, abort_flag, p.err,
+                                                  ERR_TIMEOUT_PRODUCER) &&
+                             mbar_wait<Cfg::POLL>(&empty_bar[stage], phase ^ 1u, abort_flag, p.err,
+                                                  ERR_TIMEOUT_PRODUCER)) ? 1 : 0;
+                    w = __shfl_sync(0xffffffffu, w, 0);
+                    if (!w) {
+                        ok = false;
+                        break;
                     }
-                    const int off = ((4 * h + i) ^ rx) << 4;
-                    *reinterpret_cast<uint4*>(dhi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                    if (Cfg::MODE == MODE_SPLIT)
-                        *reinterpret_cast<uint4*>(dlo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+                    // every lane observes both completed phases (lane 0 already has)
+                    while (!mbar_test_wait(&ffull_bar[fs], fphase)) {
+                    }
+                    while (!mbar_test_wait(&empty_bar[stage], phase ^ 1u)) {
+                    }
+                    tc_fence_after();   // the MMAs that read this stage's tensor memory are done
+                    const uint32_t ta = tmem_base + ((uint32_t)(tq * 32) << 16) +
+                                        (uint32_t)(Cfg::TMEM_A + stage * Cfg::TMEM_A_STAGE);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint8_t* src =
+                            fring + (size_t)fs * Cfg::F_BYTES + h * (Cfg::F_BYTES / 2) + r * 128;
+                        float4 v[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            v[i] = *reinterpret_cast<const float4*>(src + ((i ^ rx) << 4));
+                        __syncwarp();
+                        // the FP32 slot is free once every lane of the group's warps has read it
+                        if (h == 1 && lane == 0) mbar_arrive(&fempty_bar[fs]);
+                        // pairs of columns, the lower one in the lower half: hi = bf16(x) and
+                        // lo = bf16(x - hi), both rounded to nearest even (x - hi is exact)
+                        uint32_t hw[16], lw[16];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float x[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                const __nv_bfloat162 hp = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+                                hw[2 * i + j] = *reinterpret_cast<const uint32_t*>(&hp);
+                                if (Cfg::MODE == MODE_SPLIT) {
+                                    const float2 hf = __bfloat1622float2(hp);
+                                    const __nv_bfloat162 lp =
+                                        __floats2bfloat162_rn(x[2 * j] - hf.x, x[2 * j + 1] - hf.y);
+                                    lw[2 * i + j] = *reinterpret_cast<const uint32_t*>(&lp);
+                                }
+                            }
+                        }
+                        tmem_st16(ta + 16u * h, hw);
+                        if (Cfg::MODE == MODE_SPLIT) tmem_st16(ta + 32u + 16u * h, lw);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&full_bar[stage]);
                 }
-                // the tensor cores read the tiles through the async proxy
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&full_bar[stage]);
                 if (++fs == Cfg::FSTAGES) {
                     fs = 0;
                     fphase ^= 1u;
@@ -1075,7 +1180,7 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
         int acc = 0;
         uint32_t acc_phase = 0;
         bool ok = true;
-        for (int t = tile_first<PAIR>(); t < ntiles && ok; t += tile_stride<PAIR>()) {
+        for (int t = first_unit(); t < ntiles && ok; t += unit_stride()) {
             const TileInfo ti = tile_info(t);
             const int tm = ti.tm;
             // first of the 32 rows of this warp (TMEM lane quarter q of this CTA's rows)
@@ -1166,19 +1271,22 @@ __global__ void __launch_bounds__(Cfg::THREADS, 1)
                     // Two 32-column loads are in flight per wait, except for the split
                     // form's 128-column slices (a fold every 8 K blocks, off the critical path)
                     const uint64_t sc2 = f2_pack(sc, sc);
-                    constexpr int NB = (NCOL == 64 || Cfg::MODE == MODE_FP8) ? 2 : 1;
+                    constexpr int NB = ((NCOL == 64 && !Cfg::FUSED) || Cfg::MODE == MODE_FP8) ? 2 : 1;
                     // the accumulator is released as soon as the warp's last batch of
                     // columns is in registers, before that batch's FMAs
+                    const int chains = Cfg::DUAL && p.stream > 0 ? 2 : 1;
+#pragma unroll 1
+                    for (int u = 0; u < chains; ++u)
 #pragma unroll
                     for (int c0 = 0; c0 < NCOL / 32; c0 += NB) {
                         uint32_t r[NB][32];
 #pragma unroll
                         for (int c = 0; c < NB; ++c)
                             tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) +
-                                          (uint32_t)(acc * Cfg::BN + col0 + (c0 + c) * 32),
+                                          (uint32_t)(acc * Cfg::ACC_COLS + u * Cfg::BN + col0 + (c0 + c) * 32),
                                       r[c]);
                         tmem_ld_wait();
-                        if (c0 + NB >= NCOL / 32) release(acc);
+                        if (c0 + NB >= NCOL / 32 && u == chains - 1) release(acc);
 #pragma unroll
                         for (int c = 0; c < NB; ++c)
 #pragma unroll
@@ -1384,6 +1492,58 @@ __global__ void k_slice_reduce(int M, int N, const float* __restrict__ part, int
     }
 }
 
+// The pieces of the tiles that several K ranges share (see TcParams::stream), added in range
+// order: C = sum (beta = 0) or C += sum (beta = 1).  Block: `rows` rows of a 128-row tile; the
+// pieces' slots are worked out once per block (they cost 64-bit divisions), and a thread
+// has the loads of eight pieces in flight.
+static constexpr int STREAM_MAX = 512;   // most ranges of a launch (one per SM)
+template <int VEC>
+__global__ void __launch_bounds__(256) k_stream_reduce(int M, int N, int nkb, int G, long long U, int rows,
+                                                       const float* __restrict__ part, float* C, int ldc,
+                                                       int beta) {
+    __shared__ int first[STREAM_MAX];   // first row of each piece in part
+    const int per = 128 / rows, tile = blockIdx.x / per, row0 = blockIdx.x % per * rows;
+    const long long base = (long long)tile * nkb;
+    const int ga = range_of(base, G, U), np = range_of(base + nkb - 1, G, U) - ga + 1;
+    if (np > 1)
+        for (int i = threadIdx.x; i < np; i += 256)
+            first[i] = (2 * (ga + i) + (range_begin(ga + i, G, U) / nkb == tile ? 0 : 1)) * 128;
+    __syncthreads();
+    pdl_wait();
+    if (np == 1) return;   // one range covered the tile
+    const int left = min(rows, M - tile * 128 - row0), nv = N / VEC;
+    for (int i = threadIdx.x; i < left * nv; i += 256) {
+        const int r = row0 + i / nv, c = i % nv * VEC;
+        float acc[VEC], v[8][VEC];
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) acc[u] = 0.f;
+        for (int q = 0; q < np; q += 8) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (q + j < np) {
+                    const float* x = part + (size_t)(first[q + j] + r) * N + c;
+                    if (VEC == 4) {
+                        const float4 f = *reinterpret_cast<const float4*>(x);
+                        v[j][0] = f.x;
+                        v[j][1 % VEC] = f.y;
+                        v[j][2 % VEC] = f.z;
+                        v[j][3 % VEC] = f.w;
+                    } else {
+                        v[j][0] = *x;
+                    }
+                }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (q + j < np)
+#pragma unroll
+                    for (int u = 0; u < VEC; ++u) acc[u] = q + j == 0 ? v[j][u] : acc[u] + v[j][u];
+        }
+        float* cp = C + (size_t)(tile * 128 + r) * ldc + c;
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) cp[u] = beta ? cp[u] + acc[u] : acc[u];
+    }
+}
+
 // ------------------------------------------------------------ host side
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 static std::mutex g_tc_mu;
@@ -1581,8 +1741,8 @@ static const TcVariant* tc_table(int* n) {
         tcv<MODE_SPLIT3, 256, 6, true>(PGK_FAM_TC_SPLIT),
         tcv<MODE_SPLIT, 256, 3, true>(PGK_FAM_TC_SPLIT),
         // B1 = 64: A converted inside the GEMM (skinny products, N <= 64)
-        tcv<MODE_SPLIT, 64, 3, false, 2>(PGK_FAM_TC_SPLIT),
-        tcv<MODE_BF16, 64, 4, false, 3>(PGK_FAM_TC_BF16),
+        tcv<MODE_SPLIT, 64, 3, false, 5>(PGK_FAM_TC_SPLIT),
+        tcv<MODE_BF16, 64, 4, false, 5>(PGK_FAM_TC_BF16),
     };
     *n = (int)(sizeof(t) / sizeof(t[0]));
     return t;
@@ -2085,13 +2245,42 @@ static pgk_status tc_gemm_fused(const TcVariant& v, int slices, int M, int N, in
     p.beta = beta ? 1 : 0;
     p.err = device_error_word(&st);
     if (!p.err) return st;
-    // K slices: slices = 0 takes as many as fill the SMs when the 128-row tiles alone
-    // do not, each at least 8 K blocks (512) deep; every slice gets at least one K block
     const int nkb = (K + 63) / 64;
+    const long long tiles_m = ((long long)M + v.BM - 1) / v.BM;
+    const size_t piece = sizeof(float) * 128 * (size_t)N;
     if (slices == 0) {
-        const int tiles_m = (M + v.BM - 1) / v.BM;
-        slices = tiles_m < m.sm_count ? std::min(m.sm_count / tiles_m, (K + 511) / 512) : 1;
+        // K ranges: the K blocks of all tiles cut into one contiguous range per SM, at least 8
+        // blocks (512) deep, where that beats whole tiles by more than the pieces cost (about
+        // 7 blocks' time: two pieces written per CTA and the second launch)
+        const long long U = tiles_m * nkb;
+        const int G = (int)std::max(1LL, std::min<long long>(std::min(m.sm_count, STREAM_MAX), U / 8));
+        const long long whole = (tiles_m + m.sm_count - 1) / m.sm_count * nkb;
+        bool stream = G > 1 && whole > (U + G - 1) / G + 7;
+        if (stream && !workspace_ready(WS_SPLITK, 2 * G * piece)) {
+            // (a workspace cannot grow while the stream is being captured)
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+                cudaGetLastError();
+                stream = false;
+            }
+        }
+        if (stream) {
+            p.part = (float*)workspace(WS_SPLITK, 2 * G * piece, &st);
+            if (!p.part) return st;
+            p.stream = G;
+            cudaError_t e = v.launch(maps, p, G, m.sm_count, s);
+            if (e != cudaSuccess) return cuda_fail(e, "fused-conversion GEMM launch");
+            // rows per block: about one element (or four) per thread
+            const int rows = tiles_m >= m.sm_count ? 32 : 8;
+            PGK_CUDA_TRY(launch_pdl(N % 4 == 0 ? k_stream_reduce<4> : k_stream_reduce<1>,
+                                    (unsigned)(128 / rows * tiles_m), 256, 0, 1, s, M, N, nkb, G, U, rows,
+                                    (const float*)p.part, C, ldc, p.beta),
+                         "K-range reduction launch");
+            return PGK_OK;
+        }
+        slices = 1;
     }
+    // K slices: every slice gets at least one K block
     int S = std::max(1, std::min(slices, nkb));
     const int kper = (nkb + S - 1) / S;
     S = (nkb + kper - 1) / kper;
@@ -2101,7 +2290,7 @@ static pgk_status tc_gemm_fused(const TcVariant& v, int slices, int M, int N, in
         p.part = (float*)workspace(WS_SPLITK, sizeof(float) * (size_t)S * M * N, &st);
         if (!p.part) return st;
     }
-    const long long tiles = (long long)((M + v.BM - 1) / v.BM) * ((N + v.BN - 1) / v.BN) * S;
+    const long long tiles = tiles_m * ((N + v.BN - 1) / v.BN) * S;
     cudaError_t e = v.launch(maps, p, tiles, m.sm_count, s);
     if (e != cudaSuccess) return cuda_fail(e, "fused-conversion GEMM launch");
     if (S > 1) {

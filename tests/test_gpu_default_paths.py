@@ -186,3 +186,24 @@ def test_jacobi_without_parameters_in_a_graph(dev):
     ad.copy_(torch.from_numpy(a))
     g.replay()
     assert np.array_equal(ad.cpu().numpy(), stencil.jacobi(a, n, steps))
+
+
+@pytest.mark.parametrize("form", [pgk.SPLIT_BF16, pgk.BF16])
+@pytest.mark.parametrize("M,N,K", [(129, 64, 1024), (1, 1, 5000), (300, 17, 4100), (1000, 64, 1216), (20000, 7, 640),
+                                   (19500, 64, 2048), (50, 33, 40000)])
+@pytest.mark.parametrize("pad,beta", [(0, 0), (4, 1), (0, 1)])
+def test_skinny_products_over_k_ranges(dev, form, M, N, K, pad, beta):
+    """Skinny products without parameters: tiles cut into K ranges (tiles of many pieces, of
+    two, and whole ones; ragged rows, columns and K), whose pieces a second launch adds.
+    Small integers keep every sum exact, so the result equals binary64's."""
+    g = torch.Generator(device=dev).manual_seed(M + N + K)
+    lda = (K + 3) // 4 * 4 + pad
+    A, B, C0 = (torch.randint(-7, 8, (r, w), generator=g, device=dev).float()[:, :c]
+                for r, c, w in ((M, K, lda), (K, N, N + pad), (M, N, N + pad)))
+    C = torch.full((M, N + pad), float("nan"), device=dev)
+    C[:, :N] = C0
+    pgk.gemm(A, B, C[:, :N], form, beta=beta)
+    torch.cuda.synchronize()
+    pgk.check_device_error()
+    assert torch.equal(C[:, :N].double(), A.double() @ B.double() + (C0.double() if beta else 0))
+    assert torch.isnan(C[:, N:]).all()
