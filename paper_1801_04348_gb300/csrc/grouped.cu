@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "pgk_internal.cuh"
@@ -90,12 +91,16 @@ __global__ void __launch_bounds__(32, 8)
         int bm, bn;
         grouped_tile_coords(item - __ldg(prefix + lo), p.tiles_m, p.tiles_n, bm, bn);
         float* smem = reinterpret_cast<float*>(smem_gw4);
-        if (wt_vec(p.vecA, p.vecB, p.N, p.K))
-            WarpTile<Cfg, true>::run(p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, 0, p.K, bm * Cfg::BM,
-                                     bn * Cfg::BN, p.beta, p.vecC, lane, 0, smem);
-        else
-            WarpTile<Cfg, false>::run(p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, 0, p.K, bm * Cfg::BM,
-                                      bn * Cfg::BN, p.beta, p.vecC, lane, 0, smem);
+        auto tile = [&](auto va, auto vb) {
+            WarpTile<Cfg, decltype(va)::value, decltype(vb)::value>::run(
+                p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, 0, p.K, bm * Cfg::BM, bn * Cfg::BN, p.beta, p.vecC,
+                lane, 0, smem);
+        };
+        const bool va = p.vecA && p.K % 4 == 0, vb = p.vecB && p.N % 4 == 0;
+        if (va && vb) tile(std::true_type(), std::true_type());
+        else if (va) tile(std::true_type(), std::false_type());
+        else if (vb) tile(std::false_type(), std::true_type());
+        else tile(std::false_type(), std::false_type());
     }
 }
 

@@ -345,7 +345,7 @@ static cudaError_t launch_wt_program(const SimtArgs& p, int, cudaStream_t st) {
     const long long tiles =
         (long long)((p.M + Cfg::BM - 1) / Cfg::BM) * ((p.N + Cfg::BN - 1) / Cfg::BN);
     cudaError_t e;
-    const int splits = split_k(p, tiles, (const void*)k_wt<Cfg, false>, Cfg::THREADS, Cfg::SMEM, &e);
+    const int splits = split_k(p, tiles, (const void*)k_wt<Cfg, false, false>, Cfg::THREADS, Cfg::SMEM, &e);
     if (e != cudaSuccess) return e;
     if (splits < 2) return launch_wt<Cfg>(p, 1, nullptr, st);
     pgk_status ws;
@@ -435,11 +435,11 @@ void register_simt_variants(std::vector<Variant>& v) {
     add_rb<16, 16, 16, 8, 16>(v);
     add_rb<16, 16, 8, 16, 16>(v);
     // wide tiles: 128 x 128 of four warps, 64 x 64 of one warp, 32 x 32 with K slices
-    v.push_back(make_variant(PGK_FAM_RB, 8, 16, 8, 16, 8, 0, (const void*)k_wt<Wt128, false>,
+    v.push_back(make_variant(PGK_FAM_RB, 8, 16, 8, 16, 8, 0, (const void*)k_wt<Wt128, false, false>,
                              launch_wt_program<Wt128>, Wt128::SMEM));
-    v.push_back(make_variant(PGK_FAM_RB, 8, 16, 4, 8, 8, 0, (const void*)k_wt<Wt64<1>, false>,
+    v.push_back(make_variant(PGK_FAM_RB, 8, 16, 4, 8, 8, 0, (const void*)k_wt<Wt64<1>, false, false>,
                              launch_wt_program<Wt64<1>>, Wt64<1>::SMEM));
-    v.push_back(make_variant(PGK_FAM_RB, 4, 8, 4, 8, 16, 0, (const void*)k_wt<Wt32<1>, false>,
+    v.push_back(make_variant(PGK_FAM_RB, 4, 8, 4, 8, 16, 0, (const void*)k_wt<Wt32<1>, false, false>,
                              launch_wt32_program, Wt32<1>::SMEM));
 }
 

@@ -60,11 +60,13 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, int by
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
-// VEC: A and B are read 16 bytes at a time, which needs their bases and row strides on
-// 16-byte boundaries and K and N multiples of 4 (a float4 then lies wholly inside or
-// outside the matrix).  Rows and columns beyond M and N are read at the last row or
-// column instead (their outputs are never stored), K beyond its end reads as zero.
-template <class Cfg, bool VEC>
+// VA, VB: A (or B) is read 16 bytes at a time, which needs its base and row stride on
+// 16-byte boundaries and K (or N) a multiple of 4 (a float4 then lies wholly inside or
+// outside the matrix); otherwise by 4-byte asynchronous copies, lanes along the rows (along
+// K, and transposed into place without bank conflicts, for A).  Rows and columns beyond M
+// and N are read at the last row or column instead (their outputs are never stored), K
+// beyond its end reads as zero.
+template <class Cfg, bool VA, bool VB>
 struct WarpTile {
     static __device__ __forceinline__ void sync() {
         if (Cfg::NW == 1) __syncwarp();
@@ -92,23 +94,28 @@ struct WarpTile {
         constexpr int AM_STEP = Cfg::NT / (BK / 4), BK_STEP = Cfg::NT / (Cfg::BN / 4);
         static_assert(Cfg::NT % (BK / 4) == 0 && Cfg::NT % (Cfg::BN / 4) == 0, "fixed column per thread");
 
-        auto load_a = [&](int k0) {
-            const int gk = k0 + 4 * akq;
+        auto load_a = [&](int k0, int buf) {
+            if (VA) {
+                const int gk = k0 + 4 * akq;
 #pragma unroll
-            for (int i = 0; i < Cfg::LA; ++i) {
-                const int gm = min(row0 + am + i * AM_STEP, M - 1);
-                const float* p = A + (size_t)gm * lda + gk;
-                if (VEC) {
-                    ra[i] = gk < k_end ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                } else {
-                    ra[i].x = gk + 0 < k_end ? __ldg(p + 0) : 0.f;
-                    ra[i].y = gk + 1 < k_end ? __ldg(p + 1) : 0.f;
-                    ra[i].z = gk + 2 < k_end ? __ldg(p + 2) : 0.f;
-                    ra[i].w = gk + 3 < k_end ? __ldg(p + 3) : 0.f;
+                for (int i = 0; i < Cfg::LA; ++i) {
+                    const int gm = min(row0 + am + i * AM_STEP, M - 1);
+                    ra[i] = gk < k_end ? __ldg(reinterpret_cast<const float4*>(A + (size_t)gm * lda + gk))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
+            } else {
+                const int k = tid % BK, m = tid / BK;
+                const bool in = k0 + k < k_end;
+                const float* p = A + (in ? k0 + k : 0);
+                const uint32_t d = (uint32_t)__cvta_generic_to_shared(As + buf * Cfg::A_ELEMS + k * Cfg::LDAS + m);
+#pragma unroll
+                for (int i = 0; i < 4 * Cfg::LA; ++i)
+                    cp_async4(d + 4u * (uint32_t)(i * (Cfg::NT / BK)),
+                              p + (size_t)min(row0 + m + i * (Cfg::NT / BK), M - 1) * lda, in ? 4 : 0);
             }
         };
         auto store_a = [&](int buf) {
+            if (!VA) return;
             float* d0 = As + buf * Cfg::A_ELEMS + 4 * akq * Cfg::LDAS + am;
 #pragma unroll
             for (int i = 0; i < Cfg::LA; ++i) {
@@ -119,20 +126,25 @@ struct WarpTile {
                 d[3 * Cfg::LDAS] = ra[i].w;
             }
         };
-        auto load_b = [&](int k0, int buf) {
-            const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(Bs + buf * Cfg::B_ELEMS + bk * Cfg::LDBS + 4 * bnq);
-            const int gn = col0 + 4 * bnq;
+        auto load_b = [&](int k0, int buf) {   // (closes the group of copies of A, too)
+            const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(Bs + buf * Cfg::B_ELEMS);
+            if (VB) {
+                const int gn = min(col0 + 4 * bnq, N - 4);
 #pragma unroll
-            for (int i = 0; i < Cfg::LB; ++i) {
-                const int gk = k0 + bk + i * BK_STEP;
-                const bool in = gk < k_end;
-                const float* p = B + (size_t)(in ? gk : 0) * ldb;   // (nothing is read when !in)
-                const uint32_t d = d0 + 4u * (uint32_t)(i * BK_STEP * Cfg::LDBS);
-                if (VEC) {
-                    cp_async16(d, p + min(gn, N - 4), in ? 16 : 0);
-                } else {
+                for (int i = 0; i < Cfg::LB; ++i) {
+                    const int k = bk + i * BK_STEP;
+                    const bool in = k0 + k < k_end;
+                    // (nothing is read when !in)
+                    cp_async16(d0 + 4u * (uint32_t)(k * Cfg::LDBS + 4 * bnq),
+                               B + (size_t)(in ? k0 + k : 0) * ldb + gn, in ? 16 : 0);
+                }
+            } else {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) cp_async4(d + 4u * u, p + min(gn + u, N - 1), in ? 4 : 0);
+                for (int i = 0; i < 4 * Cfg::LB; ++i) {
+                    const int e = tid + i * Cfg::NT, k = e / Cfg::BN, n = e % Cfg::BN;
+                    const bool in = k0 + k < k_end;
+                    cp_async4(d0 + 4u * (uint32_t)(k * Cfg::LDBS + n),
+                              B + (size_t)(in ? k0 + k : 0) * ldb + min(col0 + n, N - 1), in ? 4 : 0);
                 }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
@@ -144,7 +156,7 @@ struct WarpTile {
 #pragma unroll
             for (int j = 0; j < Cfg::TN; ++j) acc[i][j] = 0ull;
 
-        load_a(k_begin);
+        load_a(k_begin, 0);
         load_b(k_begin, 0);
         store_a(0);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -153,7 +165,7 @@ struct WarpTile {
         for (int k0 = k_begin; k0 < k_end;) {
             const bool more = k_end - k0 > BK;
             if (more) {
-                load_a(k0 + BK);
+                load_a(k0 + BK, cur ^ 1);
                 load_b(k0 + BK, cur ^ 1);
             }
             const float* as = As + cur * Cfg::A_ELEMS + ra0;
@@ -260,7 +272,7 @@ struct WarpTile {
 // blockIdx.x: output tile; blockIdx.y: one of gridDim.y groups of KS consecutive K slices of
 // kper each.  With more than one group the partial products go to P (M x N each, in group
 // order), for a second launch to add.
-template <class Cfg, bool VEC>
+template <class Cfg, bool VA, bool VB>
 __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_wt(SimtArgs p, float* P, int kper) {
     extern __shared__ float4 smem_wt4[];
     const int tiles_m = (p.M + Cfg::BM - 1) / Cfg::BM;
@@ -271,15 +283,10 @@ __global__ void __launch_bounds__(Cfg::THREADS, Cfg::MINB) k_wt(SimtArgs p, floa
     const int kb = (int)min((long long)p.K, (long long)((int)blockIdx.y * Cfg::KS + sl) * kper);
     const int ke = kb + min(kper, p.K - kb);
     const bool split = gridDim.y > 1;
-    WarpTile<Cfg, VEC>::run(p.A, p.lda, p.B, p.ldb, split ? P + (size_t)blockIdx.y * p.M * p.N : p.C,
+    WarpTile<Cfg, VA, VB>::run(p.A, p.lda, p.B, p.ldb, split ? P + (size_t)blockIdx.y * p.M * p.N : p.C,
                             split ? p.N : p.ldc, p.M, p.N, kb, ke, bm * Cfg::BM, bn * Cfg::BN,
                             split ? 0 : p.beta, split ? (p.N & 3) == 0 : p.vecC, tid, sl,
                             reinterpret_cast<float*>(smem_wt4));
-}
-
-// Whether both operands may be read 16 bytes at a time (see WarpTile).
-__host__ __device__ inline bool wt_vec(int vecA, int vecB, int N, int K) {
-    return vecA && vecB && N % 4 == 0 && K % 4 == 0;
 }
 
 // The product as gridDim.y = groups groups of KS slices (groups > 1: P holds the partials).
@@ -291,14 +298,14 @@ static cudaError_t launch_wt(const SimtArgs& p, int groups, float* P, cudaStream
     const int slices = groups * Cfg::KS;
     const long long kper = std::min<long long>(
         INT_MAX, ((p.K + (long long)slices - 1) / slices + Cfg::BK - 1) / Cfg::BK * Cfg::BK);
-    const bool vec = wt_vec(p.vecA, p.vecB, p.N, p.K);
-    static SmemLimit limit[2];
-    const cudaError_t e = allow_smem(limit[vec], vec ? (const void*)k_wt<Cfg, true> : (const void*)k_wt<Cfg, false>,
-                                     Cfg::SMEM);
+    typedef void (*kernel)(SimtArgs, float*, int);
+    static const kernel kernels[4] = {k_wt<Cfg, false, false>, k_wt<Cfg, true, false>, k_wt<Cfg, false, true>,
+                                      k_wt<Cfg, true, true>};
+    static SmemLimit limit[4];
+    const int i = (p.vecA && p.K % 4 == 0 ? 1 : 0) + (p.vecB && p.N % 4 == 0 ? 2 : 0);
+    const cudaError_t e = allow_smem(limit[i], (const void*)kernels[i], Cfg::SMEM);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)tiles, (unsigned)groups);
-    if (vec) k_wt<Cfg, true><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);
-    else k_wt<Cfg, false><<<grid, Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);
+    kernels[i]<<<dim3((unsigned)tiles, (unsigned)groups), Cfg::THREADS, Cfg::SMEM, st>>>(p, P, (int)kper);
     return cudaGetLastError();
 }
 
