@@ -60,26 +60,31 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::MINB)
     }
 }
 
-// The same on single-warp 64 x 64 tiles of simt_warp.cuh, eight to an SM.  Bound by the
-// FMA pipe and by what a tile wastes on ragged edges, where 64 x 64 loses less than
-// 128-wide tiles; the next item is taken, and its problem searched for by the whole warp
-// (32 prefix sums at a time), before the current tile runs.
-__global__ void __launch_bounds__(32, 8)
+// The same on the single-warp 64 x 64 tiles of simt_warp.cuh, or on KS warps per tile that
+// share its K, eight warps to an SM.  Bound by the FMA pipe and by what a tile wastes on
+// ragged edges, where 64 x 64 loses less than 128-wide tiles; the next item is taken, and its
+// problem searched for by the whole warp (32 prefix sums at a time), before the current tile
+// runs.  With few tiles the longest K is what a group takes: see grouped_default.
+template <int KS>
+__global__ void __launch_bounds__(32 * KS, 8 / KS)
     k_grouped_wt(const GProb* __restrict__ probs, const int* __restrict__ prefix, int G, int total,
                  int* counter) {
-    typedef Wt64<1> Cfg;
     extern __shared__ float4 smem_gw4[];
-    const int lane = threadIdx.x;
-    auto take = [&] {
-        int i = 0;
-        if (lane == 0) i = atomicAdd(counter, 1);
-        return i;   // valid in lane 0
-    };
-    int next = take();
+    __shared__ int s_next;
+    const int lane = threadIdx.x & 31;
+    int next = 0;
+    if (threadIdx.x == 0) next = atomicAdd(counter, 1);
     for (;;) {
-        const int item = __shfl_sync(0xffffffffu, next, 0);
+        int item;
+        if (KS == 1) {
+            item = __shfl_sync(0xffffffffu, next, 0);
+        } else {
+            if (threadIdx.x == 0) s_next = next;
+            __syncthreads();
+            item = s_next;
+        }
         if (item >= total) break;
-        next = take();
+        if (threadIdx.x == 0) next = atomicAdd(counter, 1);
         int lo = 0, hi = G;   // the problem lies in [lo, hi): the largest g with prefix[g] <= item
         while (hi - lo > 1) {
             const int step = (hi - lo + 31) / 32, g = lo + lane * step;
@@ -90,17 +95,16 @@ __global__ void __launch_bounds__(32, 8)
         const GProb p = probs[lo];
         int bm, bn;
         grouped_tile_coords(item - __ldg(prefix + lo), p.tiles_m, p.tiles_n, bm, bn);
+        typedef Wt64<KS> Cfg;
+        const int sl = threadIdx.x >> 5, kper = ((p.K + KS - 1) / KS + Cfg::BK - 1) / Cfg::BK * Cfg::BK;
+        const int kb = min(p.K, sl * kper), ke = min(p.K, kb + kper);
         float* smem = reinterpret_cast<float*>(smem_gw4);
-        auto tile = [&](auto va, auto vb) {
-            WarpTile<Cfg, decltype(va)::value, decltype(vb)::value>::run(
-                p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, 0, p.K, bm * Cfg::BM, bn * Cfg::BN, p.beta, p.vecC,
-                lane, 0, smem);
-        };
-        const bool va = p.vecA && p.K % 4 == 0, vb = p.vecB && p.N % 4 == 0;
-        if (va && vb) tile(std::true_type(), std::true_type());
-        else if (va) tile(std::true_type(), std::false_type());
-        else if (vb) tile(std::false_type(), std::true_type());
-        else tile(std::false_type(), std::false_type());
+        if (p.vecA && p.vecB && p.K % 4 == 0 && p.N % 4 == 0)
+            WarpTile<Cfg, true, true>::run(p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, kb, ke, bm * Cfg::BM,
+                                           bn * Cfg::BN, p.beta, p.vecC, lane, sl, smem);
+        else
+            WarpTile<Cfg, false, false>::run(p.A, p.lda, p.B, p.ldb, p.C, p.ldc, p.M, p.N, kb, ke, bm * Cfg::BM,
+                                             bn * Cfg::BN, p.beta, p.vecC, lane, sl, smem);
     }
 }
 
@@ -109,6 +113,7 @@ struct GroupedVariant {
     int bm, bn, smem, threads;
     const void* func;
     cudaError_t (*launch)(const GProb*, const int*, int, int, int*, int grid, cudaStream_t);
+    int ks;   // K slices of a tile (warps), 1 for the programs
 };
 
 template <class Cfg>
@@ -118,17 +123,26 @@ static cudaError_t launch_grouped(const GProb* t, const int* prefix, int G, int 
     return cudaGetLastError();
 }
 
+template <int KS>
 static cudaError_t launch_grouped_wt(const GProb* t, const int* prefix, int G, int total, int* counter,
                                      int grid, cudaStream_t st) {
-    k_grouped_wt<<<grid, Wt64<1>::THREADS, Wt64<1>::SMEM, st>>>(t, prefix, G, total, counter);
+    k_grouped_wt<KS><<<grid, Wt64<KS>::THREADS, Wt64<KS>::SMEM, st>>>(t, prefix, G, total, counter);
     return cudaGetLastError();
+}
+
+template <int KS>
+static GroupedVariant gv_wt() {
+    typedef Wt64<KS> Cfg;
+    GroupedVariant v = {4, 8, 16, 8, 8, Cfg::BM, Cfg::BN, Cfg::SMEM, Cfg::THREADS,
+                        (const void*)k_grouped_wt<KS>, launch_grouped_wt<KS>, KS};
+    return v;
 }
 
 template <int B0, int B1, int SR, int S, int BK>
 static GroupedVariant gv() {
     typedef RbCfg<B0, B1, SR, S, BK> Cfg;
     GroupedVariant v = {B0, B1, SR, S, BK, Cfg::BM, Cfg::BN, Cfg::SMEM, Cfg::NT,
-                        (const void*)k_grouped<Cfg>, launch_grouped<Cfg>};
+                        (const void*)k_grouped<Cfg>, launch_grouped<Cfg>, 1};
     return v;
 }
 
@@ -137,8 +151,7 @@ static const GroupedVariant* grouped_table(int* n) {
         gv<16, 16, 8, 8, 8>(),  gv<16, 16, 8, 8, 16>(), gv<16, 16, 4, 4, 8>(),
         gv<16, 16, 8, 4, 8>(),  gv<16, 16, 4, 8, 8>(),  gv<8, 16, 8, 8, 8>(),
         gv<16, 8, 8, 8, 8>(),   gv<8, 8, 8, 8, 8>(),
-        {4, 8, 16, 8, 8, Wt64<1>::BM, Wt64<1>::BN, Wt64<1>::SMEM, Wt64<1>::THREADS,
-         (const void*)k_grouped_wt, launch_grouped_wt},
+        gv_wt<1>(),
     };
     *n = (int)(sizeof(t) / sizeof(t[0]));
     return t;
@@ -247,6 +260,41 @@ static const GroupedVariant* find_grouped(const pgk_params* prog) {
     return nullptr;
 }
 
+// The variant of a group without parameters: 64 x 64 tiles with as many K slices (warps) as
+// give the smallest estimate: the work spread over the SMs' eight warps each, or the longest
+// tile if that is more, and half a longest tile for the uneven end.  A K step of a tile costs a warp 304 cycles beside a second one on its scheduler, a
+// tile 6000 more (its problem, first loads and stores), and K slices meet at 256 cycles each.
+// Measured: 512 problems up to 2048 a side take one slice, 1.97 ms (64 x 64 tiles of 256
+// threads: 4.05); ten of them, 823 tiles, 72 us (one slice 345, 256 threads 145).  Where most of the work reads unaligned rows and there
+// are tiles for every warp, the 128 x 64 tiles of 128 threads are faster (512 problems of odd
+// sizes: 2.59 ms against 3.55): they copy half as many elements per product.
+static const GroupedVariant* grouped_default(int G, const pgk_problem* pr, int sms) {
+    static const GroupedVariant t[] = {gv_wt<1>(), gv_wt<2>(), gv_wt<4>(), gv_wt<8>()};
+    double tiles = 0, steps = 0, unaligned = 0, longest = 0;
+    for (int i = 0; i < G; ++i) {
+        const double n = (double)((pr[i].M + 63LL) / 64) * (double)((pr[i].N + 63LL) / 64);
+        tiles += n;
+        steps += n * pr[i].K;
+        if (!al16(pr[i].A) || !al16(pr[i].B) || pr[i].lda % 4 || pr[i].ldb % 4 || pr[i].K % 4 || pr[i].N % 4)
+            unaligned += n * pr[i].K;
+        longest = std::max(longest, (double)pr[i].K);
+    }
+    const pgk_params wide = {16, 8, 8, 8, 8};
+    if (2 * unaligned > steps && tiles >= 8.0 * sms) return find_grouped(&wide);
+    const GroupedVariant* best = &t[0];
+    double best_t = 0;
+    for (const GroupedVariant& v : t) {
+        const double fixed = 6000 + (v.ks > 1 ? 300 + 256.0 * v.ks : 0);
+        const double last = longest * 304 / v.ks + fixed;
+        const double est = std::max((steps * 304 + tiles * v.ks * fixed) / (8.0 * sms), last) + 0.5 * last;
+        if (&v == t || est < best_t) {
+            best = &v;
+            best_t = est;
+        }
+    }
+    return best;
+}
+
 static pgk_status grid_for(const GroupedVariant& v, int total, int* grid) {
     pgk_machine m;
     pgk_status st = current_machine(&m, NULL);
@@ -295,17 +343,19 @@ extern "C" pgk_status pgk_gemm_grouped(int G, const pgk_problem* problems, pgk_d
         set_error("the grouped GEMM runs the FP32 SIMT family and the tensor-core forms");
         return PGK_ERR_UNSUPPORTED;
     }
-    pgk_params p;
-    if (prog) {
-        p = *prog;
-    } else if (pgk_tune_cache_get(-G, 0, 0, PGK_F32, &p) != PGK_OK) {
-        pgk_params d = {4, 8, 8, 16, 8};
-        p = d;
-    }
-    const GroupedVariant* v = find_grouped(&p);
-    if (!v) {
-        set_error("no grouped variant (B0=%d B1=%d s=%d sr=%d tile=%d)", p.B0, p.B1, p.s, p.sr, p.tile);
-        return PGK_ERR_UNSUPPORTED;
+    pgk_params p = {4, 8, 8, 16, 8};
+    const GroupedVariant* v = nullptr;
+    if (prog || pgk_tune_cache_get(-G, 0, 0, PGK_F32, &p) == PGK_OK) {
+        if (prog) p = *prog;
+        v = find_grouped(&p);
+        if (!v) {
+            set_error("no grouped variant (B0=%d B1=%d s=%d sr=%d tile=%d)", p.B0, p.B1, p.s, p.sr, p.tile);
+            return PGK_ERR_UNSUPPORTED;
+        }
+    } else {
+        pgk_machine m;
+        if ((st = current_machine(&m, NULL)) != PGK_OK) return st;
+        v = grouped_default(G, problems, m.sm_count);
     }
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<unsigned char> img;
@@ -325,7 +375,7 @@ extern "C" pgk_status pgk_gemm_grouped(int G, const pgk_problem* problems, pgk_d
     int dev = 0;
     PGK_CUDA_TRY(cudaGetDevice(&dev), "cudaGetDevice");
     std::vector<long long> key;
-    key.reserve(9 * (size_t)G + 9);
+    key.reserve(9 * (size_t)G + 10);
     key.push_back(dev);
     key.push_back(G);
     key.push_back(p.B0);
@@ -334,6 +384,7 @@ extern "C" pgk_status pgk_gemm_grouped(int G, const pgk_problem* problems, pgk_d
     key.push_back(p.sr);
     key.push_back(p.tile);
     key.push_back(beta);
+    key.push_back(v->ks);
     for (int i = 0; i < G; ++i) {
         const pgk_problem& q = problems[i];
         key.push_back(q.M);

@@ -211,32 +211,53 @@ struct WarpTile {
                            : make_float4(lo32(acc[i / 2][4 * j]), lo32(acc[i / 2][4 * j + 1]),
                                          lo32(acc[i / 2][4 * j + 2]), lo32(acc[i / 2][4 * j + 3]));
         };
+        auto load4 = [&](int gm, int gn) {   // C there, zero outside
+            const float* cp = C + (size_t)gm * ldc + gn;
+            float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (gm >= M) return c;
+            if (vecC && gn + 3 < N) return *reinterpret_cast<const float4*>(cp);
+            if (gn + 0 < N) c.x = cp[0];
+            if (gn + 1 < N) c.y = cp[1];
+            if (gn + 2 < N) c.z = cp[2];
+            if (gn + 3 < N) c.w = cp[3];
+            return c;
+        };
         auto store4 = [&](float4 o, int gm, int gn) {
             float* cp = C + (size_t)gm * ldc + gn;
+            if (gm >= M) return;
             if (vecC && gn + 3 < N) {
-                if (beta) {
-                    const float4 c = *reinterpret_cast<const float4*>(cp);
-                    o.x += c.x;
-                    o.y += c.y;
-                    o.z += c.z;
-                    o.w += c.w;
-                }
                 *reinterpret_cast<float4*>(cp) = o;
             } else {
-                if (gn + 0 < N) cp[0] = beta ? cp[0] + o.x : o.x;
-                if (gn + 1 < N) cp[1] = beta ? cp[1] + o.y : o.y;
-                if (gn + 2 < N) cp[2] = beta ? cp[2] + o.z : o.z;
-                if (gn + 3 < N) cp[3] = beta ? cp[3] + o.w : o.w;
+                if (gn + 0 < N) cp[0] = o.x;
+                if (gn + 1 < N) cp[1] = o.y;
+                if (gn + 2 < N) cp[2] = o.z;
+                if (gn + 3 < N) cp[3] = o.w;
             }
         };
         if (Cfg::KS == 1) {
+            // with beta = 1, two rows of C are read before the first is written (four spill in
+            // the grouped kernel)
+            constexpr int NJ = Cfg::TN / 4, RB = 2;
 #pragma unroll
-            for (int i = 0; i < Cfg::TM; ++i) {
-                const int gm = row0 + ra0 + (i / 4) * 4 * Cfg::LM + i % 4;
-                if (gm < M) {
+            for (int i0 = 0; i0 < Cfg::TM; i0 += RB) {
+                float4 c[RB][NJ];
+                if (beta) {
 #pragma unroll
-                    for (int j = 0; j < Cfg::TN / 4; ++j) store4(out4(i, j), gm, col0 + cb0 + j * 4 * Cfg::LN);
+                    for (int i = 0; i < RB; ++i)
+#pragma unroll
+                        for (int j = 0; j < NJ; ++j)
+                            c[i][j] = load4(row0 + ra0 + (i0 + i) / 4 * 4 * Cfg::LM + (i0 + i) % 4,
+                                            col0 + cb0 + j * 4 * Cfg::LN);
                 }
+#pragma unroll
+                for (int i = 0; i < RB; ++i)
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j) {
+                        float4 o = out4(i0 + i, j);
+                        if (beta) o = make_float4(o.x + c[i][j].x, o.y + c[i][j].y, o.z + c[i][j].z, o.w + c[i][j].w);
+                        store4(o, row0 + ra0 + (i0 + i) / 4 * 4 * Cfg::LM + (i0 + i) % 4,
+                               col0 + cb0 + j * 4 * Cfg::LN);
+                    }
             }
             return;
         }
@@ -252,20 +273,31 @@ struct WarpTile {
                 *reinterpret_cast<float4*>(part + r * Cfg::BN + cb0 + j * 4 * Cfg::LN) = out4(i, j);
         }
         __syncthreads();
-        for (int e = sl * Cfg::NT + tid; e < Cfg::BM * Cfg::BN / 4; e += Cfg::THREADS) {
-            const int r = e / (Cfg::BN / 4), c = e % (Cfg::BN / 4) * 4;
-            if (row0 + r >= M || col0 + c >= N) continue;
-            float4 s = *reinterpret_cast<const float4*>(smem + 4 * e);
+        constexpr int EB = Cfg::BM * Cfg::BN / 4 / Cfg::THREADS < 4 ? Cfg::BM * Cfg::BN / 4 / Cfg::THREADS : 4;
+        static_assert(Cfg::KS == 1 || Cfg::BM * Cfg::BN / 4 % (EB * Cfg::THREADS) == 0, "whole batches");
+        for (int e0 = sl * Cfg::NT + tid; e0 < Cfg::BM * Cfg::BN / 4; e0 += EB * Cfg::THREADS) {
+            float4 c[EB];
+            if (beta) {
 #pragma unroll
-            for (int y = 1; y < Cfg::KS; ++y) {
-                const float4 v = *reinterpret_cast<const float4*>(smem + y * (Cfg::BM * Cfg::BN) + 4 * e);
-                s.x += v.x;
-                s.y += v.y;
-                s.z += v.z;
-                s.w += v.w;
+                for (int q = 0; q < EB; ++q) {
+                    const int e = e0 + q * Cfg::THREADS;
+                    c[q] = load4(row0 + e / (Cfg::BN / 4), col0 + e % (Cfg::BN / 4) * 4);
+                }
             }
-            store4(s, row0 + r, col0 + c);
+#pragma unroll
+            for (int q = 0; q < EB; ++q) {
+                const int e = e0 + q * Cfg::THREADS;
+                float4 s = *reinterpret_cast<const float4*>(smem + 4 * e);
+#pragma unroll
+                for (int y = 1; y < Cfg::KS; ++y) {
+                    const float4 v = *reinterpret_cast<const float4*>(smem + y * (Cfg::BM * Cfg::BN) + 4 * e);
+                    s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
+                }
+                if (beta) s = make_float4(s.x + c[q].x, s.y + c[q].y, s.z + c[q].z, s.w + c[q].w);
+                store4(s, row0 + e / (Cfg::BN / 4), col0 + e % (Cfg::BN / 4) * 4);
+            }
         }
+        __syncthreads();   // the partial tiles are read: shared memory may be used again
     }
 };
 
