@@ -187,9 +187,35 @@ __device__ __forceinline__ float4 load_row4(const float* __restrict__ src, int l
     return v;
 }
 
-__device__ __forceinline__ uint32_t e4m3(float x, float scale) {
-    // binary32 division rounded to nearest, then E4M3 round to nearest even, saturated
-    return (uint32_t)__nv_cvt_float_to_fp8(__fdiv_rn(x, scale), __NV_SATFINITE, __NV_E4M3);
+// Codes of x / scale: the quotient rounded to nearest in binary32, then E4M3 round to
+// nearest even, saturated, two values per conversion.  The quotient comes from the correctly
+// rounded reciprocal y of the scale: q = x y, then twice q + (x - q scale) y.  The first step
+// leaves q within an ulp, and the second then rounds correctly while nothing under- or
+// overflows (P. Markstein, IBM Journal of Research and Development 34, 1990); quotients that
+// do underflow give the code of a zero with the sign of x either way.  `fast` is false for
+// scales so small or large that the reciprocal or a product could leave the normal range,
+// and for scales that are not finite: those divide.
+struct Quotient {
+    float scale, y;
+    bool fast;
+    __device__ __forceinline__ float operator()(float x) const {
+        if (!fast) return __fdiv_rn(x, scale);
+        float q = __fmul_rn(x, y);
+        q = __fmaf_rn(__fmaf_rn(-q, scale, x), y, q);
+        q = __fmaf_rn(__fmaf_rn(-q, scale, x), y, q);
+        return copysignf(q, x);
+    }
+    __device__ __forceinline__ uint32_t two(float x0, float x1) const {
+        return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2((*this)(x0), (*this)(x1)), __NV_SATFINITE,
+                                                  __NV_E4M3);
+    }
+};
+__device__ __forceinline__ Quotient make_quotient(float s) {
+    Quotient q;
+    q.scale = s;
+    q.y = __frcp_rn(s);
+    q.fast = s >= 0x1p-90f && s <= 0x1p90f;
+    return q;
 }
 
 // Writes the four codes of word w (byte k = element k) to dst + off, or the
@@ -205,12 +231,18 @@ __device__ __forceinline__ void store_codes(uint8_t* __restrict__ dst, size_t of
 }
 
 // Per-tile FP8 quantisation: one block of QUANT_THREADS per 128 x 128 tile.  The
-// tile is read from global memory once, into registers: warp w, lane l holds rows
-// 16 i + w, columns 4 l .. 4 l + 3 (each warp load is one 512-byte row segment).
+// tile is read from global memory once, into registers: warp w holds rows 16 i + w;
+// lane l columns 4 l .. 4 l + 3 (each warp load is one 512-byte row segment), or, where
+// the source does not allow 128-bit loads, columns l, l + 32, l + 64, l + 96.
 // The block's amax gives the scale.  Row output: each warp writes 128 contiguous
 // bytes of a row.  Transposed output: the codes go through a shared tile with a
 // row pitch of 129 bytes (conflict-free both for the row-wise stores and for the
 // column-wise reads), and each warp writes whole 128-byte rows of the transpose.
+// Both operands of a product go in one launch.  Bound by the loads of two blocks an SM, which
+// their arithmetic does not overlap (4.8 TB/s at 8192^2, the reciprocal and the paired
+// conversions gain nothing there); sources without 128-bit loads, which read four
+// neighbouring columns a lane, 82 -> 70 us at 8191 x 8193; FP8 8192 x 1024 x 4096 93.4 -> 90.8 us
+// a call.
 static constexpr int QUANT_THREADS = 512;
 static constexpr int QUANT_PITCH = 129;
 
@@ -230,17 +262,29 @@ __device__ __forceinline__ int grouped_item_problem(const int* __restrict__ pref
 // (rows mode) or transposed for source rows below wbound (the K extent; entries
 // between the source size and wbound are the codes of zeros).  Called by every
 // thread of a QUANT_THREADS block; red and tile are the block's shared buffers.
-template <bool TRANS>
+template <bool TRANS, bool VEC>
 __device__ __forceinline__ void quant_tile(const float* __restrict__ src, int lds, int rows, int cols,
                                            int wbound, int r0, int c0, uint8_t* __restrict__ dst,
-                                           int ldd, float* scale_out, int vec_in, int vec_out,
+                                           int ldd, float* scale_out, int vec_out,
                                            float* red, uint8_t* tile) {
     constexpr int WARPS = QUANT_THREADS / 32;          // 16
     constexpr int NV = 128 * 128 / 4 / QUANT_THREADS;  // float4 per thread: 8
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float4 v[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) v[i] = load_row4(src, lds, rows, cols, r0 + i * WARPS + warp, c0 + lane * 4, vec_in);
+    for (int i = 0; i < NV; ++i) {
+        const int r = r0 + i * WARPS + warp;
+        if (VEC) {
+            v[i] = load_row4(src, lds, rows, cols, r, c0 + lane * 4, 1);
+        } else {
+            const int c = c0 + lane;
+            const float* p = src + (size_t)r * lds + c;
+            v[i].x = r < rows && c < cols ? __ldg(p) : 0.f;
+            v[i].y = r < rows && c + 32 < cols ? __ldg(p + 32) : 0.f;
+            v[i].z = r < rows && c + 64 < cols ? __ldg(p + 64) : 0.f;
+            v[i].w = r < rows && c + 96 < cols ? __ldg(p + 96) : 0.f;
+        }
+    }
     // amax (|x| is exact and max is order independent; out-of-range elements are 0)
     float amax = 0.f;
 #pragma unroll
@@ -256,16 +300,24 @@ __device__ __forceinline__ void quant_tile(const float* __restrict__ src, int ld
     for (int w = 1; w < WARPS; ++w) amax = fmaxf(amax, red[w]);
     const float scale = amax == 0.f ? 1.f : __fdiv_rn(amax, 448.f);
     if (threadIdx.x == 0) *scale_out = scale;
+    const Quotient quot = make_quotient(scale);
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-        const int rr = i * WARPS + warp, cc = lane * 4;   // position in the tile
-        const uint32_t w = e4m3(v[i].x, scale) | (e4m3(v[i].y, scale) << 8) |
-                           (e4m3(v[i].z, scale) << 16) | (e4m3(v[i].w, scale) << 24);
+        const int rr = i * WARPS + warp;   // row in the tile
+        const uint32_t w = quot.two(v[i].x, v[i].y) | (quot.two(v[i].z, v[i].w) << 16);
         if (TRANS) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tile[rr * QUANT_PITCH + cc + k] = (uint8_t)(w >> (8 * k));
+            for (int k = 0; k < 4; ++k)
+                tile[rr * QUANT_PITCH + (VEC ? 4 * lane + k : lane + 32 * k)] = (uint8_t)(w >> (8 * k));
         } else if (r0 + rr < rows) {
-            store_codes(dst, (size_t)(r0 + rr) * ldd + c0 + cc, w, min(4, wbound - c0 - cc), vec_out);
+            uint8_t* d = dst + (size_t)(r0 + rr) * ldd + c0;
+            if (VEC) {
+                store_codes(d, 4 * lane, w, min(4, wbound - c0 - 4 * lane), vec_out);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (c0 + lane + 32 * k < wbound) d[lane + 32 * k] = (uint8_t)(w >> (8 * k));
+            }
         }
     }
     if (TRANS) {
@@ -287,18 +339,39 @@ __device__ __forceinline__ void quant_tile(const float* __restrict__ src, int ld
     }
 }
 
+// One operand of a quantisation launch: `items` 128 x 128 tiles (zero: none), `tile_cols` of
+// them along a row of the source.
+struct QuantOp {
+    const float* src;
+    uint8_t* dst;
+    float* scales;
+    int lds, ldd, ld_scales, rows, cols;
+    int vec_in, vec_out;
+    int items, tile_cols;
+};
+
 template <bool TRANS>
-__global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8(int rows, int cols,
-                                                             const float* __restrict__ src, int lds,
-                                                             uint8_t* __restrict__ dst, int ldd,
-                                                             float* __restrict__ scales, int ld_scales,
-                                                             int vec_in, int vec_out) {
+__device__ __forceinline__ void quant_item(const QuantOp& q, int item, float* red, uint8_t* tile) {
+    const int ti = item / q.tile_cols, tj = item % q.tile_cols;
+    float* so = q.scales + (size_t)ti * q.ld_scales + tj;
+    const int wb = TRANS ? q.rows : q.cols;
+    if (q.vec_in)
+        quant_tile<TRANS, true>(q.src, q.lds, q.rows, q.cols, wb, ti * 128, tj * 128, q.dst, q.ldd, so, q.vec_out,
+                                red, tile);
+    else
+        quant_tile<TRANS, false>(q.src, q.lds, q.rows, q.cols, wb, ti * 128, tj * 128, q.dst, q.ldd, so, q.vec_out,
+                                 red, tile);
+}
+
+// Operand a (rows kept) takes the first a.items blocks, operand b (transposed) the rest:
+// both operands of a product in one launch.
+__global__ void __launch_bounds__(QUANT_THREADS, 2) k_quant_fp8(const QuantOp a, const QuantOp b) {
     __shared__ float red[QUANT_THREADS / 32];
-    __shared__ uint8_t tile[TRANS ? 128 * QUANT_PITCH : 1];
+    __shared__ uint8_t tile[128 * QUANT_PITCH];
     pdl_wait();
-    quant_tile<TRANS>(src, lds, rows, cols, TRANS ? rows : cols, blockIdx.y * 128, blockIdx.x * 128,
-                      dst, ldd, scales + (size_t)blockIdx.y * ld_scales + blockIdx.x, vec_in, vec_out,
-                      red, tile);
+    const int i = blockIdx.x;
+    if (i < a.items) quant_item<false>(a, i, red, tile);
+    else quant_item<true>(b, i - a.items, red, tile);
     pdl_trigger();
 }
 
@@ -327,8 +400,12 @@ __global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8_grouped(const GQuan
         const int ti = local / tcols, tj = local % tcols;
         float* so = TRANS ? scales + (size_t)ti * ld_scales + q.scale_off + tj
                           : scales + (size_t)(q.scale_off + ti) * ld_scales + tj;
-        quant_tile<TRANS>(q.src, q.lds, q.rows, q.cols, q.width, ti * 128, tj * 128,
-                          dst + (size_t)q.dst_row * ldd, (int)ldd, so, q.vec, 1, red, tile);
+        if (q.vec)
+            quant_tile<TRANS, true>(q.src, q.lds, q.rows, q.cols, q.width, ti * 128, tj * 128,
+                                    dst + (size_t)q.dst_row * ldd, (int)ldd, so, 1, red, tile);
+        else
+            quant_tile<TRANS, false>(q.src, q.lds, q.rows, q.cols, q.width, ti * 128, tj * 128,
+                                     dst + (size_t)q.dst_row * ldd, (int)ldd, so, 1, red, tile);
         __syncthreads();   // red is reused by the next item
     }
     pdl_trigger();
@@ -403,19 +480,45 @@ pgk_status launch_cvt_operands(int mode, int M, int N, int K, const float* A, in
     return launch_cvt_ops(mode, op[0], op[1], st);
 }
 
-pgk_status launch_quant_fp8(int rows, int cols, const float* src, int lds, uint8_t* dst, int ldd,
-                            float* scales, int ld_scales, int transpose, cudaStream_t st) {
-    dim3 grid((cols + 127) / 128, (rows + 127) / 128);
-    if (grid.y > 65535) {
+static bool quant_op(QuantOp* o, int rows, int cols, const float* src, int lds, uint8_t* dst, int ldd,
+                     float* scales, int ld_scales) {
+    const long long tr = ((long long)rows + 127) / 128, tc = ((long long)cols + 127) / 128;
+    if (tr > 65535) {
         set_error("too many rows for FP8 quantisation");
-        return PGK_ERR_INVALID_ARG;
+        return false;
     }
-    const int vec_in = aligned(src, 16) && lds % 4 == 0;
-    const int vec_out = aligned(dst, 4) && ldd % 4 == 0;
-    PGK_CUDA_TRY(launch_pdl(transpose ? k_quant_fp8<true> : k_quant_fp8<false>, grid, QUANT_THREADS, 0, 1, st, rows,
-                            cols, src, lds, dst, ldd, scales, ld_scales, vec_in, vec_out),
+    if (tr * tc > INT_MAX / 2) {
+        set_error("matrix too large for one quantisation launch");
+        return false;
+    }
+    *o = QuantOp{src, dst, scales, lds, ldd, ld_scales, rows, cols, aligned(src, 16) && lds % 4 == 0,
+                 aligned(dst, 4) && ldd % 4 == 0, (int)(tr * tc), (int)tc};
+    return true;
+}
+
+static pgk_status launch_quant_ops(const QuantOp& a, const QuantOp& b, cudaStream_t st) {
+    PGK_CUDA_TRY(launch_pdl(k_quant_fp8, (unsigned)a.items + (unsigned)b.items, QUANT_THREADS, 0, 1, st, a, b),
                  "FP8 quantisation launch");
     return PGK_OK;
+}
+
+static pgk_status launch_quant_fp8(int rows, int cols, const float* src, int lds, uint8_t* dst, int ldd,
+                                   float* scales, int ld_scales, int transpose, cudaStream_t st) {
+    QuantOp op[2];
+    memset(op, 0, sizeof(op));
+    if (!quant_op(&op[transpose ? 1 : 0], rows, cols, src, lds, dst, ldd, scales, ld_scales))
+        return PGK_ERR_INVALID_ARG;
+    return launch_quant_ops(op[0], op[1], st);
+}
+
+// Both operands of a product, A (M x K) and, unless b is NULL, B (K x N) transposed: one launch.
+pgk_status launch_quant_operands(int M, int N, int K, const float* A, int lda, uint8_t* a, float* sa,
+                                 const float* B, int ldb, uint8_t* b, float* sb, int Kp, cudaStream_t st) {
+    QuantOp op[2];
+    memset(op, 0, sizeof(op));
+    if (!quant_op(&op[0], M, K, A, lda, a, Kp, sa, (K + 127) / 128)) return PGK_ERR_INVALID_ARG;
+    if (b && !quant_op(&op[1], K, N, B, ldb, b, Kp, sb, (N + 127) / 128)) return PGK_ERR_INVALID_ARG;
+    return launch_quant_ops(op[0], op[1], st);
 }
 
 // ------------------------------------------------------ grouped conversion

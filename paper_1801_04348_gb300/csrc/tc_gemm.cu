@@ -2197,8 +2197,8 @@ pgk_status tc_gemm_grouped(int G, const pgk_problem* pr, pgk_dtype dtype, const 
 pgk_status launch_cvt_operands(int mode, int M, int N, int K, const float* A, int lda, uint16_t* a0,
                                uint16_t* a1, const float* B, int ldb, uint16_t* b0, uint16_t* b1, int Kp,
                                cudaStream_t st);
-pgk_status launch_quant_fp8(int rows, int cols, const float* src, int lds, uint8_t* dst, int ldd,
-                            float* scales, int ld_scales, int transpose, cudaStream_t st);
+pgk_status launch_quant_operands(int M, int N, int K, const float* A, int lda, uint8_t* a, float* sa,
+                                 const float* B, int ldb, uint8_t* b, float* sb, int Kp, cudaStream_t st);
 
 // The fused-conversion programs: B^T is prepared (BF16, or hi and lo) into a
 // library workspace, A is read in FP32 by the kernel itself.
@@ -2340,8 +2340,8 @@ pgk_status tc_gemm_fp32_inputs(const pgk_case& c, int M, int N, int K, pgk_dtype
     if (!sa) return st;
     float* sb = (float*)workspace(WS_SB, (size_t)kt * nt * 4, &st);
     if (!sb) return st;
-    if ((st = launch_quant_fp8(M, K, A, lda, (uint8_t*)a0, Kp, sa, kt, 0, s)) != PGK_OK) return st;
-    if (prep_b && (st = launch_quant_fp8(K, N, B, ldb, (uint8_t*)b0, Kp, sb, nt, 1, s)) != PGK_OK)
+    if ((st = launch_quant_operands(M, N, K, A, lda, (uint8_t*)a0, sa, B, ldb, prep_b ? (uint8_t*)b0 : nullptr, sb,
+                                    Kp, s)) != PGK_OK)
         return st;
     return tc_gemm_launch(c, M, N, K, dtype, a0, Kp, b0, Kp, nullptr, nullptr, sa, sb, C, ldc, beta,
                           s);

@@ -207,3 +207,36 @@ def test_skinny_products_over_k_ranges(dev, form, M, N, K, pad, beta):
     pgk.check_device_error()
     assert torch.equal(C[:, :N].double(), A.double() @ B.double() + (C0.double() if beta else 0))
     assert torch.isnan(C[:, N:]).all()
+
+
+@pytest.mark.parametrize("R,Cc", [(128, 128), (5, 300), (257, 131), (640, 384)])
+@pytest.mark.parametrize("kind", ["ties", "tiny", "huge", "specials"])
+def test_fp8_codes_bit_exact_on_hard_tiles(dev, R, Cc, kind):
+    """Tiles whose quotients lie on or beside the midpoints of E4M3, scales too small or too
+    large for the reciprocal (which divide), signed zeros and quotients that underflow; both
+    layouts, sources with and without 128-bit loads, against the oracle's codes and scales."""
+    from oracle import quant
+    rng = np.random.default_rng(R + Cc)
+    if kind == "ties":     # amax 448 s: quotients k / 16, one ulp to either side
+        X = (rng.integers(-7168, 7169, (R, Cc)) / 16).astype(np.float32)
+        X = np.nextafter(X, np.where(rng.random((R, Cc)) < 0.5, -np.inf, np.inf).astype(np.float32),
+                         where=rng.random((R, Cc)) < 0.6, out=X.copy())
+        X[::128, ::128] = 448.0
+        X *= np.float32(3.0) ** rng.integers(-8, 8)
+    else:
+        X = inputs.normal((R, Cc), 3) * np.float32({"tiny": 1e-37, "huge": 1e36, "specials": 1.0}[kind])
+    if kind in ("tiny", "specials"):
+        X[rng.random((R, Cc)) < 0.2] = -0.0
+        X[rng.random((R, Cc)) < 0.2] *= np.float32(1e-5)
+        X[rng.random((R, Cc)) < 0.1] = np.float32(1e-42)
+    codes, S = quant.fp8_tile_quant(X)
+    for pad in (0, 1):
+        W = torch.zeros(R, (Cc + 3) // 4 * 4 + pad, device=dev)
+        W[:, :Cc] = torch.from_numpy(X)
+        q = torch.zeros(R, (Cc + 15) // 16 * 16, dtype=torch.uint8, device=dev)
+        s = torch.zeros((R + 127) // 128, (Cc + 127) // 128, device=dev)
+        pgk.quant_fp8(W[:, :Cc], q, s, 0)
+        assert np.array_equal(s.cpu().numpy(), S) and np.array_equal(q.cpu().numpy()[:, :Cc], codes)
+        qt = torch.zeros(Cc, (R + 15) // 16 * 16, dtype=torch.uint8, device=dev)
+        pgk.quant_fp8(W[:, :Cc], qt, s, 1)
+        assert np.array_equal(qt.cpu().numpy()[:, :R], codes.T)
