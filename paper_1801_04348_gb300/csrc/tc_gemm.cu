@@ -1748,14 +1748,13 @@ static const TcVariant* tc_table(int* n) {
     return t;
 }
 
-// What a tile of each program costs a launch without parameters (us on GB300, at full
-// load): per K block (64 deep, FP8 128) and once per round of tiles.  From the launches
-// alone of 2048^3, 4096^3, 8192^3, 8192 x 1024 x 4096 and 3000 x 3000 x 500; the estimate
-// is within 10 % of them.
+// What a launch of each program costs without parameters (us on GB300, at full load): per
+// K block (64 deep, FP8 128), per round of tiles and once.
 struct TcCost {
     pgk_dtype dtype;
     int BM, BN, stages;
-    float block, round;
+    // us of a K block, of a K block in a round of column halves, of a tile, of a launch
+    float block, half, round, start;
     // K-split launch of the same tiles, if there is one
     int (*clusters)(int slices);
     tc_launch_fn ksplit;
@@ -1763,18 +1762,17 @@ struct TcCost {
 template <int MODE, int BN, int ST>
 static TcCost tc_cost(pgk_dtype dtype, float block, float round) {
     typedef TcCfg<MODE, BN, ST> Cfg;
-    return TcCost{dtype, 128, BN, ST, block, round, ksplit_clusters<Cfg>, launch_ksplit<Cfg>};
+    return TcCost{dtype, 128, BN, ST, block, 0.f, round, 0.f, ksplit_clusters<Cfg>, launch_ksplit<Cfg>};
 }
 static const TcCost* tc_costs(int* n) {
     static const TcCost t[] = {
         tc_cost<MODE_SPLIT, 128, 3>(PGK_SPLIT_BF16, 0.60f, 2.5f),
-        {PGK_SPLIT_BF16, 128, 256, 2, 1.05f, 3.5f, nullptr, nullptr},
-        {PGK_SPLIT_BF16, 256, 256, 3, 0.90f, 7.0f, nullptr, nullptr},
-        tc_cost<MODE_BF16, 128, 6>(PGK_BF16, 0.333f, 2.5f),
-        {PGK_BF16, 128, 256, 4, 0.41f, 3.0f, nullptr, nullptr},
-        {PGK_BF16, 256, 256, 6, 0.34f, 4.5f, nullptr, nullptr},
+        {PGK_SPLIT_BF16, 256, 256, 3, 0.90f, 0.60f, 5.3f, 2.7f, nullptr, nullptr},
+        tc_cost<MODE_BF16, 128, 6>(PGK_BF16, 0.28f, 2.5f),
+        {PGK_BF16, 128, 256, 4, 0.40f, 0.33f, 2.5f, -0.5f, nullptr, nullptr},
+        {PGK_BF16, 256, 256, 6, 0.307f, 0.28f, 3.0f, 1.15f, nullptr, nullptr},
         tc_cost<MODE_FP8, 128, 6>(PGK_FP8_E4M3, 0.47f, 2.5f),
-        {PGK_FP8_E4M3, 128, 256, 4, 0.68f, 3.0f, nullptr, nullptr},
+        {PGK_FP8_E4M3, 128, 256, 4, 0.68f, 0.f, 3.0f, 0.f, nullptr, nullptr},
     };
     *n = (int)(sizeof(t) / sizeof(t[0]));
     return t;
@@ -1782,10 +1780,15 @@ static const TcCost* tc_costs(int* n) {
 
 // The tile program and K slices of a call without parameters: the smallest estimate over
 // the form's programs.  A launch takes ceil(tiles / places) rounds (a last round at most
-// half full runs as column halves in half the time, BF16 and split 256-wide tiles); where
-// 128 x 128 tiles leave places idle, clusters of 2 to 8 K slices (as many as can be resident
-// at once: 76 of two, 15 of eight) share their K blocks at 3 us for the exchange.  Against one fixed program per form: split 8192^3 2020 -> 1630 us a
-// launch (CTA pairs), FP8 8192 x 1024 x 4096 66 -> 49 (256-wide tiles).
+// half full runs as column halves, BF16 and split 256-wide tiles); where 128 x 128 tiles
+// leave places idle, clusters of 2 to 8 K slices (as many as can be resident at once: 76 of
+// two, 15 of eight) share their K blocks at 3 us for the exchange.  The constants fit timed
+// calls of all programs over 850 shapes from 32 to 16384 a side: without K slices the
+// planned program is 0.3 % (split) and 1.2 % (BF16) above the fastest one on average, where
+// one fixed program per form is 2.0 % (128 x 128 x 3) and 1.9 % (128 x 256 x 4) above it.
+// Split 128 x 256 tiles are never ahead of both others by more than 2 % and are not planned.
+// Against one fixed program per form: split 8192^3 2020 -> 1630 us a launch (CTA pairs),
+// FP8 8192 x 1024 x 4096 66 -> 49 (256-wide tiles).
 static void tc_plan(const pgk_machine& m, int M, int N, int K, pgk_dtype dtype, pgk_params* p, int* slices) {
     int n;
     const TcCost* t = tc_costs(&n);
@@ -1798,9 +1801,10 @@ static void tc_plan(const pgk_machine& m, int M, int N, int K, pgk_dtype dtype, 
             (((long long)M + t[i].BM - 1) / t[i].BM) * (((long long)N + t[i].BN - 1) / t[i].BN);
         const long long places = t[i].BM == 256 ? m.sm_count / 2 : m.sm_count;
         const long long rem = tiles % places;
-        double rounds = (double)((tiles + places - 1) / places);
-        if (t[i].BN == 256 && dtype != PGK_FP8_E4M3 && rem > 0 && 2 * rem <= places) rounds -= 0.5;
-        const double est = rounds * (nkb * t[i].block + t[i].round);
+        const bool halves = t[i].half > 0.f && rem > 0 && 2 * rem <= places;
+        const double rounds = (double)((tiles + places - 1) / places);
+        const double est = t[i].start + rounds * (nkb * t[i].block + t[i].round) -
+                           (halves ? nkb * (t[i].block - t[i].half) : 0.f);
         if (!any || est < best) {
             any = true;
             best = est;
