@@ -444,10 +444,11 @@ PGK_API pgk_status pgk_mlp_adam(int count, float* theta, const float* grad, floa
 
 /* Time each candidate (host array of ncand pgk_params; NULL = the built-in
  * feasible set of the form) for C = A*B on the given device buffers (C is
- * overwritten), `reps` timed runs each after one warm-up, CUDA events on
- * `stream`.  ms_out (host, ncand entries, may be NULL) gets each candidate's
- * median time, +inf if infeasible.  The fastest feasible candidate is written
- * to *best and stored in the tuning cache used by pgk_gemm(prog = NULL).
+ * overwritten), `reps` timed runs each after one warm-up (a run is one call, or
+ * up to 32 calls of less than 0.1 ms), CUDA events on `stream`.  ms_out (host,
+ * ncand entries, may be NULL) gets each candidate's median time, +inf if
+ * infeasible.  The fastest feasible candidate is written to *best and stored
+ * in the tuning cache used by pgk_gemm(prog = NULL).
  * If log_path is not NULL one CSV row per candidate is appended there.
  * Synchronises `stream`.  Errors: INVALID_ARG, INFEASIBLE (none feasible), CUDA. */
 PGK_API pgk_status pgk_autotune(int M, int N, int K, pgk_dtype dtype, const float* A, int lda,

@@ -510,10 +510,14 @@ pgk_status pgk_autotune(int M, int N, int K, pgk_dtype dtype, const float* A, in
         st = pgk_select_case(&m, M, N, K, dtype, &cand[i], &c);
         if (st == PGK_OK) {
             st = pgk_gemm(M, N, K, dtype, A, lda, B, ldb, C, ldc, 0, &cand[i], stream);  // warm-up
+            // a run is one call, or as many as take about 0.2 ms: events resolve a microsecond
+            // or two, several percent of a small product
             std::vector<float> t;
+            int calls = 1;
             for (int r = 0; r < reps && st == PGK_OK; ++r) {
                 cudaEventRecord(e0, s);
-                st = pgk_gemm(M, N, K, dtype, A, lda, B, ldb, C, ldc, 0, &cand[i], stream);
+                for (int q = 0; q < calls && st == PGK_OK; ++q)
+                    st = pgk_gemm(M, N, K, dtype, A, lda, B, ldb, C, ldc, 0, &cand[i], stream);
                 cudaEventRecord(e1, s);
                 if (st != PGK_OK) break;
                 cudaError_t e = cudaEventSynchronize(e1);
@@ -523,7 +527,12 @@ pgk_status pgk_autotune(int M, int N, int K, pgk_dtype dtype, const float* A, in
                 }
                 float x = 0.f;
                 cudaEventElapsedTime(&x, e0, e1);
-                t.push_back(x);
+                if (calls == 1 && x < 0.1f) {   // too short: time runs of several calls instead
+                    calls = x > 0.2f / 32 ? (int)ceilf(0.2f / x) : 32;
+                    --r;
+                    continue;
+                }
+                t.push_back(x / calls);
             }
             if (st == PGK_OK && !t.empty()) {
                 std::sort(t.begin(), t.end());
