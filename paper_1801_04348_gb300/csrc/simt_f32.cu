@@ -279,10 +279,15 @@ struct WtPlan {
 // side, ragged and unaligned ones) the estimate's choice is within 10 % of the fastest;
 // 256^3 runs in 6.2 us (64 x 64 tiles of 256 threads: 14.4), 1024^3 in 47 (94 without
 // slices), 2048^3 in 283 (331 with 128 x 128 tiles, 256 of them on 304 places).
+// Rows of C off the 16-byte boundaries are written 4 bytes a lane, and the warps of a 128 x
+// 128 tile do so at once where eight single-warp tiles take turns: 2000 cycles a block more.
+// 4384 x 1565 x 48 takes 24.7 us in 64 x 64 tiles and 28.3 in 128 x 128 ones, 3417 x 2576 x
+// 609 takes 264 and 246.
 // More than one group needs a workspace, shared per device, which short products never
 // used: it is limited to K >= 4096 with few tiles, where every program splits K, and left
 // out while the stream is being captured (a workspace cannot grow there).
-static WtPlan wt_plan(int M, int N, int K, int sms, bool groups_allowed, int tile) {
+static WtPlan wt_plan(const SimtArgs& p, int sms, bool groups_allowed, int tile) {
+    const int M = p.M, N = p.N, K = p.K;
     WtPlan best = {nullptr, 1};
     double best_t = 0;
     const long long t64 = (long long)((M + 63) / 64) * ((N + 63) / 64);
@@ -298,6 +303,7 @@ static WtPlan wt_plan(int M, int N, int K, int sms, bool groups_allowed, int til
             const double resident = k.tile == 32 ? 4 : 2;   // warps per scheduler (registers)
             double t = steps * (per_sched <= 1 ? k.alone : k.shared * per_sched) +
                        2000 * ceil(per_sched / resident);
+            if (k.tile == 128 && !p.vecC) t += 2000 * blocks;
             if (k.ks > 1) t += blocks * (k.ks * k.tile * k.tile / 16 + 300);
             if (g > 1) t += 9000 + (double)g * M * N * 8 / 3400;
             if (!best.kind || t < best_t) {
@@ -328,12 +334,12 @@ static cudaError_t run_wt(const SimtArgs& p, const WtPlan& plan, cudaStream_t st
 cudaError_t simt_wide_launch(const SimtArgs& p, int tile, cudaStream_t st) {
     pgk_machine m;
     if (current_machine(&m, NULL) != PGK_OK) return cudaErrorInvalidDevice;
-    WtPlan plan = wt_plan(p.M, p.N, p.K, m.sm_count, true, tile);
+    WtPlan plan = wt_plan(p, m.sm_count, true, tile);
     if (plan.groups > 1) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
             cudaGetLastError();
-            plan = wt_plan(p.M, p.N, p.K, m.sm_count, false, tile);
+            plan = wt_plan(p, m.sm_count, false, tile);
         }
     }
     return run_wt(p, plan, st);
