@@ -6,6 +6,7 @@
 // tensor-core kernels read.  All are HBM-bound streaming kernels.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
+#include <float.h>
 #include <string.h>
 
 #include <algorithm>
@@ -189,33 +190,42 @@ __device__ __forceinline__ float4 load_row4(const float* __restrict__ src, int l
 
 // Codes of x / scale: the quotient rounded to nearest in binary32, then E4M3 round to
 // nearest even, saturated, two values per conversion.  The quotient comes from the correctly
-// rounded reciprocal y of the scale: q = x y, then twice q + (x - q scale) y.  The first step
+// rounded reciprocal y of the scale: q = x y, then twice q - (q scale - x) y.  The first step
 // leaves q within an ulp, and the second then rounds correctly while nothing under- or
 // overflows (P. Markstein, IBM Journal of Research and Development 34, 1990); quotients that
-// do underflow give the code of a zero with the sign of x either way.  `fast` is false for
-// scales so small or large that the reciprocal or a product could leave the normal range,
-// and for scales that are not finite: those divide.
+// do underflow give the code of a zero with the sign of x either way, and a zero x keeps its
+// sign.  Scales outside [2^-90, 2^90], where the reciprocal or a product could leave the
+// normal range, are brought into it together with x: see quotient_prescale.
 struct Quotient {
     float scale, y;
-    bool fast;
     __device__ __forceinline__ float operator()(float x) const {
-        if (!fast) return __fdiv_rn(x, scale);
         float q = __fmul_rn(x, y);
-        q = __fmaf_rn(__fmaf_rn(-q, scale, x), y, q);
-        q = __fmaf_rn(__fmaf_rn(-q, scale, x), y, q);
-        return copysignf(q, x);
+        q = __fmaf_rn(-__fmaf_rn(q, scale, -x), y, q);
+        q = __fmaf_rn(-__fmaf_rn(q, scale, -x), y, q);
+        return q;
     }
     __device__ __forceinline__ uint32_t two(float x0, float x1) const {
         return (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2((*this)(x0), (*this)(x1)), __NV_SATFINITE,
                                                   __NV_E4M3);
     }
+    __device__ __forceinline__ uint32_t four(float4 x) const {
+        return __byte_perm(two(x.x, x.y), two(x.z, x.w), 0x5410);
+    }
 };
-__device__ __forceinline__ Quotient make_quotient(float s) {
-    Quotient q;
-    q.scale = s;
-    q.y = __frcp_rn(s);
-    q.fast = s >= 0x1p-90f && s <= 0x1p90f;
-    return q;
+__device__ __forceinline__ bool quotient_in_range(float s) { return s >= 0x1p-90f && s <= 0x1p90f; }
+// For a scale out of range: the factor of x, and the scale that then divides it.  Powers of
+// two keep the quotient's bits (an x that underflows has the code of a zero with its sign
+// anyway).  A scale of zero or infinity leaves x / s to the factor: infinities, which become
+// values beyond the largest code, zeros of either sign and NaN.
+__device__ __forceinline__ float quotient_prescale(float s, float* divisor) {
+    const bool edge = s == 0.f || s > FLT_MAX;
+    const float m = edge ? __frcp_rn(s) : s < 1.f ? 0x1p64f : 0x1p-64f;
+    *divisor = edge ? 1.f : s * m;
+    return m;
+}
+__device__ __forceinline__ float prescaled(float x, float m) {
+    const float t = x * m;
+    return m > FLT_MAX && fabsf(t) > FLT_MAX ? copysignf(1024.f, t) : t;
 }
 
 // Writes the four codes of word w (byte k = element k) to dst + off, or the
@@ -230,21 +240,24 @@ __device__ __forceinline__ void store_codes(uint8_t* __restrict__ dst, size_t of
     for (int k = 0; k < n; ++k) dst[off + k] = (uint8_t)(w >> (8 * k));
 }
 
-// Per-tile FP8 quantisation: one block of QUANT_THREADS per 128 x 128 tile.  The
-// tile is read from global memory once, into registers: warp w holds rows 16 i + w;
-// lane l columns 4 l .. 4 l + 3 (each warp load is one 512-byte row segment), or, where
-// the source does not allow 128-bit loads, columns l, l + 32, l + 64, l + 96.
-// The block's amax gives the scale.  Row output: each warp writes 128 contiguous
-// bytes of a row.  Transposed output: the codes go through a shared tile with a
-// row pitch of 129 bytes (conflict-free both for the row-wise stores and for the
-// column-wise reads), and each warp writes whole 128-byte rows of the transpose.
-// Both operands of a product go in one launch.  Bound by the loads of two blocks an SM, which
-// their arithmetic does not overlap (4.8 TB/s at 8192^2, the reciprocal and the paired
-// conversions gain nothing there); sources without 128-bit loads, which read four
-// neighbouring columns a lane, 82 -> 70 us at 8191 x 8193; FP8 8192 x 1024 x 4096 93.4 -> 90.8 us
-// a call.
+// Per-tile FP8 quantisation: blocks of QUANT_THREADS, a 128 x 128 tile at a time, read from
+// global memory once into registers: a warp holds eight rows (quant_row), lane l columns 4 l ..
+// 4 l + 3 (each warp load is one 512-byte row segment), or, where the source does not allow
+// 128-bit loads, columns l, l + 32, l + 64, l + 96.  The block's amax gives the scale.  Row
+// output: each warp writes 128 contiguous bytes of a row.  Transposed output: four rows of a
+// column become one word, the words go through a swizzled shared tile (quant_slot), and each
+// warp writes whole 128-byte rows of the transpose.
+// Both operands of a product go in one launch.  Where a block gets several tiles, the next
+// one is copied to shared memory while this one is quantised, each thread into slots that
+// only it reads.  With the loads covered it is bound by instruction issue: of 23 instructions
+// an element, addresses, bounds and the sign and range of each quotient were over half.
+// Measured on GB300 at 8192^2 (one tile a block, a branch and a sign copy a quotient, byte
+// stores to the shared tile): 69.9 -> 56.0 us kept (6.0 TB/s), 69.8 -> 65 transposed; FP8
+// 8192 x 1024 x 4096 90.0 -> 82.4 us a call; 100 grouped problems of up to 1024 144.8 -> 136.1.
+// Sources without 128-bit loads, 4-byte loads one tile a block, take 71 to 76 us at 8191 x 8193.
 static constexpr int QUANT_THREADS = 512;
-static constexpr int QUANT_PITCH = 129;
+static constexpr int QUANT_TILE_WORDS = 128 * 32;
+static constexpr int QUANT_STAGE_BYTES = 128 * 128 * 4;
 
 // Problem of a grouped work item: the largest g with prefix[g] <= item.
 __device__ __forceinline__ int grouped_item_problem(const int* __restrict__ prefix, int G, int item) {
@@ -257,23 +270,21 @@ __device__ __forceinline__ int grouped_item_problem(const int* __restrict__ pref
     return lo;
 }
 
-// One 128 x 128 tile at (r0, c0) of src (rows x cols, zero outside): its scale goes
-// to *scale_out, its codes to dst, in the source layout for columns below wbound
-// (rows mode) or transposed for source rows below wbound (the K extent; entries
-// between the source size and wbound are the codes of zeros).  Called by every
-// thread of a QUANT_THREADS block; red and tile are the block's shared buffers.
+// Row i of a warp: eight consecutive rows where four of them become one word of a column,
+// every 16th row otherwise (the 16 warps then read 16 neighbouring rows at a time).
+__device__ __forceinline__ int quant_row(bool trans, int warp, int i) {
+    return trans ? 128 / (QUANT_THREADS / 32) * warp + i : QUANT_THREADS / 32 * i + warp;
+}
+
+// The thread's part of the 128 x 128 tile at (r0, c0) of src (rows x cols), zero outside.
+static constexpr int QUANT_NV = 128 * 128 / 4 / QUANT_THREADS;   // float4 per thread: 8
 template <bool TRANS, bool VEC>
-__device__ __forceinline__ void quant_tile(const float* __restrict__ src, int lds, int rows, int cols,
-                                           int wbound, int r0, int c0, uint8_t* __restrict__ dst,
-                                           int ldd, float* scale_out, int vec_out,
-                                           float* red, uint8_t* tile) {
-    constexpr int WARPS = QUANT_THREADS / 32;          // 16
-    constexpr int NV = 128 * 128 / 4 / QUANT_THREADS;  // float4 per thread: 8
+__device__ __forceinline__ void quant_load(float4 (&v)[QUANT_NV], const float* __restrict__ src, int lds,
+                                           int rows, int cols, int r0, int c0) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float4 v[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int r = r0 + i * WARPS + warp;
+    for (int i = 0; i < QUANT_NV; ++i) {
+        const int r = r0 + quant_row(TRANS, warp, i);
         if (VEC) {
             v[i] = load_row4(src, lds, rows, cols, r, c0 + lane * 4, 1);
         } else {
@@ -285,6 +296,48 @@ __device__ __forceinline__ void quant_tile(const float* __restrict__ src, int ld
             v[i].w = r < rows && c + 96 < cols ? __ldg(p + 96) : 0.f;
         }
     }
+}
+
+// The same as asynchronous copies into the thread's own slots of `stage`.
+__device__ __forceinline__ void quant_prefetch(float4* stage, bool trans, const float* __restrict__ src,
+                                               int lds, int rows, int cols, int r0, int c0) {
+    const int warp = threadIdx.x >> 5, r = r0 + quant_row(trans, warp, 0), c = c0 + (threadIdx.x & 31) * 4;
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(stage + threadIdx.x);
+    // (nothing is read when n is zero)
+    const int n = 4 * max(0, min(4, cols - c));
+    const float* p = src + (n ? (size_t)r * lds + c : 0);
+    const int step = quant_row(trans, warp, 1) - quant_row(trans, warp, 0);
+    const size_t pitch = n ? (size_t)step * lds : 0;
+    const bool whole = r0 + 128 <= rows;
+#pragma unroll
+    for (int i = 0; i < QUANT_NV; ++i) {
+        const bool in = whole || r + i * step < rows;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + i * QUANT_THREADS * 16),
+                     "l"(in ? p : src), "r"(in ? n : 0)
+                     : "memory");
+        p += pitch;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Word of the shared tile that holds rows 4 q .. 4 q + 3 of a column: conflict-free for lanes
+// on consecutive q, on consecutive columns and on every fourth column.
+__device__ __forceinline__ int quant_slot(int col, int q) {
+    return col * 32 + (q ^ (col >> 2) ^ ((col & 3) << 3));
+}
+
+// Quantises a tile loaded by quant_load or quant_prefetch: its scale goes to *scale_out, its
+// codes to dst, in the source layout for columns below wbound (rows mode) or transposed for
+// source rows below wbound (the K extent; entries between the source size and wbound are the
+// codes of zeros).  Called by every thread of a QUANT_THREADS block; red and tile are the
+// block's shared buffers; next() runs when every value has been read.
+template <bool TRANS, bool VEC, class Next>
+__device__ __forceinline__ void quant_tile(float4 (&v)[QUANT_NV], int rows, int cols, int wbound, int r0,
+                                           int c0, uint8_t* __restrict__ dst, int ldd, float* scale_out,
+                                           int vec_out, float* red, uint32_t* tile, Next next) {
+    constexpr int WARPS = QUANT_THREADS / 32;          // 16
+    constexpr int NV = QUANT_NV;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // amax (|x| is exact and max is order independent; out-of-range elements are 0)
     float amax = 0.f;
 #pragma unroll
@@ -294,46 +347,68 @@ __device__ __forceinline__ void quant_tile(const float* __restrict__ src, int ld
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if (lane == 0) red[warp] = amax;
+    next();
     __syncthreads();
     amax = red[0];
 #pragma unroll
     for (int w = 1; w < WARPS; ++w) amax = fmaxf(amax, red[w]);
     const float scale = amax == 0.f ? 1.f : __fdiv_rn(amax, 448.f);
     if (threadIdx.x == 0) *scale_out = scale;
-    const Quotient quot = make_quotient(scale);
+    float divisor = scale;
+    if (!quotient_in_range(scale)) {
+        const float m = quotient_prescale(scale, &divisor);
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int rr = i * WARPS + warp;   // row in the tile
-        const uint32_t w = quot.two(v[i].x, v[i].y) | (quot.two(v[i].z, v[i].w) << 16);
-        if (TRANS) {
+        for (int i = 0; i < NV; ++i)
+            v[i] = make_float4(prescaled(v[i].x, m), prescaled(v[i].y, m), prescaled(v[i].z, m),
+                               prescaled(v[i].w, m));
+    }
+    const Quotient quot = {divisor, __frcp_rn(divisor)};
+    uint32_t w[NV];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                tile[rr * QUANT_PITCH + (VEC ? 4 * lane + k : lane + 32 * k)] = (uint8_t)(w >> (8 * k));
-        } else if (r0 + rr < rows) {
-            uint8_t* d = dst + (size_t)(r0 + rr) * ldd + c0;
-            if (VEC) {
-                store_codes(d, 4 * lane, w, min(4, wbound - c0 - 4 * lane), vec_out);
-            } else {
+    for (int i = 0; i < NV; ++i) w[i] = quot.four(v[i]);
+    if (!TRANS) {
+        const int r = r0 + warp;
+        uint8_t* d = dst + (size_t)r * ldd + c0;
+        const bool whole = VEC && vec_out && r0 + 128 <= rows && c0 + 128 <= wbound;
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (c0 + lane + 32 * k < wbound) d[lane + 32 * k] = (uint8_t)(w >> (8 * k));
+        for (int i = 0; i < NV; ++i, d += (size_t)WARPS * ldd) {
+            if (whole) {
+                *reinterpret_cast<uint32_t*>(d + 4 * lane) = w[i];
+            } else if (r + WARPS * i < rows) {
+                if (VEC) {
+                    store_codes(d, 4 * lane, w[i], min(4, wbound - c0 - 4 * lane), vec_out);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (c0 + lane + 32 * k < wbound) d[lane + 32 * k] = (uint8_t)(w[i] >> (8 * k));
+                }
             }
         }
-    }
-    if (TRANS) {
+    } else {
+#pragma unroll
+        for (int h = 0; h < NV / 4; ++h) {
+            // four rows of four columns to four columns of four rows
+            const uint32_t p0 = __byte_perm(w[4 * h], w[4 * h + 1], 0x5140);
+            const uint32_t p1 = __byte_perm(w[4 * h + 2], w[4 * h + 3], 0x5140);
+            const uint32_t p2 = __byte_perm(w[4 * h], w[4 * h + 1], 0x7362);
+            const uint32_t p3 = __byte_perm(w[4 * h + 2], w[4 * h + 3], 0x7362);
+            const uint32_t t[4] = {__byte_perm(p0, p1, 0x5410), __byte_perm(p0, p1, 0x7632),
+                                   __byte_perm(p2, p3, 0x5410), __byte_perm(p2, p3, 0x7632)};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                tile[quant_slot(VEC ? 4 * lane + k : lane + 32 * k, NV / 4 * warp + h)] = t[k];
+        }
         __syncthreads();
         // output row j of the tile = source column c0 + j; lane l writes source rows
         // r0 + 4 l .. r0 + 4 l + 3 of it
+        const int j0 = warp * (128 / WARPS), n = min(4, wbound - r0 - 4 * lane);
+        uint8_t* d = dst + (size_t)(c0 + j0) * ldd + r0 + 4 * lane;
+        const bool whole = vec_out && c0 + 128 <= cols && r0 + 128 <= wbound;
 #pragma unroll
-        for (int jj = 0; jj < 128 / WARPS; ++jj) {
-            const int j = warp * (128 / WARPS) + jj;
-            if (c0 + j >= cols) break;
-            const uint8_t* col = tile + (4 * lane) * QUANT_PITCH + j;
-            const uint32_t w = (uint32_t)col[0] | ((uint32_t)col[QUANT_PITCH] << 8) |
-                               ((uint32_t)col[2 * QUANT_PITCH] << 16) |
-                               ((uint32_t)col[3 * QUANT_PITCH] << 24);
-            store_codes(dst, (size_t)(c0 + j) * ldd + r0 + 4 * lane, w, min(4, wbound - r0 - 4 * lane),
-                        vec_out);
+        for (int j = 0; j < 128 / WARPS; ++j, d += ldd) {
+            const uint32_t x = tile[quant_slot(j0 + j, lane)];
+            if (whole) *reinterpret_cast<uint32_t*>(d) = x;
+            else if (c0 + j0 + j < cols) store_codes(d, 0, x, n, vec_out);
         }
         __syncthreads();   // the shared tile may be reused by the block's next tile
     }
@@ -350,28 +425,62 @@ struct QuantOp {
     int items, tile_cols;
 };
 
-template <bool TRANS>
-__device__ __forceinline__ void quant_item(const QuantOp& q, int item, float* red, uint8_t* tile) {
+template <bool TRANS, bool VEC, class Next>
+__device__ __forceinline__ void quant_item(float4 (&v)[QUANT_NV], const QuantOp& q, int item, float* red,
+                                           uint32_t* tile, Next next) {
     const int ti = item / q.tile_cols, tj = item % q.tile_cols;
-    float* so = q.scales + (size_t)ti * q.ld_scales + tj;
-    const int wb = TRANS ? q.rows : q.cols;
-    if (q.vec_in)
-        quant_tile<TRANS, true>(q.src, q.lds, q.rows, q.cols, wb, ti * 128, tj * 128, q.dst, q.ldd, so, q.vec_out,
-                                red, tile);
-    else
-        quant_tile<TRANS, false>(q.src, q.lds, q.rows, q.cols, wb, ti * 128, tj * 128, q.dst, q.ldd, so, q.vec_out,
-                                 red, tile);
+    quant_tile<TRANS, VEC>(v, q.rows, q.cols, TRANS ? q.rows : q.cols, ti * 128, tj * 128, q.dst, q.ldd,
+                           q.scales + (size_t)ti * q.ld_scales + tj, q.vec_out, red, tile, next);
 }
 
-// Operand a (rows kept) takes the first a.items blocks, operand b (transposed) the rest:
-// both operands of a product in one launch.
+// Items [0, a.items) are the tiles of operand a (rows kept), the rest those of operand b
+// (transposed): both operands of a product in one launch, at most two blocks an SM, each over
+// every gridDim.x-th item.
 __global__ void __launch_bounds__(QUANT_THREADS, 2) k_quant_fp8(const QuantOp a, const QuantOp b) {
-    __shared__ float red[QUANT_THREADS / 32];
-    __shared__ uint8_t tile[128 * QUANT_PITCH];
+    extern __shared__ float4 stage[];   // QUANT_STAGE_BYTES
+    __shared__ float red[2][QUANT_THREADS / 32];
+    __shared__ uint32_t tile[QUANT_TILE_WORDS];
     pdl_wait();
-    const int i = blockIdx.x;
-    if (i < a.items) quant_item<false>(a, i, red, tile);
-    else quant_item<true>(b, i - a.items, red, tile);
+    const int total = a.items + b.items;
+    auto fetch = [&](int i) {
+        if (i >= total) return;
+        const bool tr = i >= a.items;
+        if (!(tr ? b.vec_in : a.vec_in)) return;
+        const int j = tr ? i - a.items : i, w = tr ? b.tile_cols : a.tile_cols;
+        quant_prefetch(stage, tr, tr ? b.src : a.src, tr ? b.lds : a.lds, tr ? b.rows : a.rows,
+                       tr ? b.cols : a.cols, j / w * 128, j % w * 128);
+    };
+    int buf = 0;
+    for (int i = blockIdx.x; i < total; i += gridDim.x, buf ^= 1) {
+        const bool tr = i >= a.items;
+        const int j = tr ? i - a.items : i;
+        const bool first = i == (int)blockIdx.x;   // loaded as it is needed
+        auto next = [&] {
+            if (!first) fetch(i + gridDim.x);
+        };
+        float4 v[QUANT_NV];
+        if (tr ? b.vec_in : a.vec_in) {
+            if (first) {
+                if (tr) quant_load<true, true>(v, b.src, b.lds, b.rows, b.cols, j / b.tile_cols * 128,
+                                               j % b.tile_cols * 128);
+                else quant_load<false, true>(v, a.src, a.lds, a.rows, a.cols, j / a.tile_cols * 128,
+                                             j % a.tile_cols * 128);
+                fetch(i + gridDim.x);
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+                for (int k = 0; k < QUANT_NV; ++k) v[k] = stage[k * QUANT_THREADS + threadIdx.x];
+            }
+            if (tr) quant_item<true, true>(v, b, j, red[buf], tile, next);
+            else quant_item<false, true>(v, a, j, red[buf], tile, next);
+        } else if (tr) {
+            quant_load<true, false>(v, b.src, b.lds, b.rows, b.cols, j / b.tile_cols * 128, j % b.tile_cols * 128);
+            quant_item<true, false>(v, b, j, red[buf], tile, next);
+        } else {
+            quant_load<false, false>(v, a.src, a.lds, a.rows, a.cols, j / a.tile_cols * 128, j % a.tile_cols * 128);
+            quant_item<false, false>(v, a, j, red[buf], tile, next);
+        }
+    }
     pdl_trigger();
 }
 
@@ -381,15 +490,11 @@ __global__ void __launch_bounds__(QUANT_THREADS, 2) k_quant_fp8(const QuantOp a,
 // along K), its tile scales to scales + scale_off with row stride ld_scales (A:
 // one row per 128-row block, B: one row per 128-deep K chunk).
 template <bool TRANS>
-__global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8_grouped(const GQuant* __restrict__ probs,
-                                                                     const int* __restrict__ prefix,
-                                                                     int G, int total,
-                                                                     uint8_t* __restrict__ dst,
-                                                                     long long ldd,
-                                                                     float* __restrict__ scales,
-                                                                     int ld_scales) {
+__global__ void __launch_bounds__(QUANT_THREADS, 2)
+    k_quant_fp8_grouped(const GQuant* __restrict__ probs, const int* __restrict__ prefix, int G, int total,
+                        uint8_t* __restrict__ dst, long long ldd, float* __restrict__ scales, int ld_scales) {
     __shared__ float red[QUANT_THREADS / 32];
-    __shared__ uint8_t tile[TRANS ? 128 * QUANT_PITCH : 1];
+    __shared__ uint32_t tile[TRANS ? QUANT_TILE_WORDS : 1];
     pdl_wait();
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int g = grouped_item_problem(prefix, G, item);
@@ -400,12 +505,17 @@ __global__ void __launch_bounds__(QUANT_THREADS) k_quant_fp8_grouped(const GQuan
         const int ti = local / tcols, tj = local % tcols;
         float* so = TRANS ? scales + (size_t)ti * ld_scales + q.scale_off + tj
                           : scales + (size_t)(q.scale_off + ti) * ld_scales + tj;
-        if (q.vec)
-            quant_tile<TRANS, true>(q.src, q.lds, q.rows, q.cols, q.width, ti * 128, tj * 128,
-                                    dst + (size_t)q.dst_row * ldd, (int)ldd, so, 1, red, tile);
-        else
-            quant_tile<TRANS, false>(q.src, q.lds, q.rows, q.cols, q.width, ti * 128, tj * 128,
-                                     dst + (size_t)q.dst_row * ldd, (int)ldd, so, 1, red, tile);
+        uint8_t* d = dst + (size_t)q.dst_row * ldd;
+        float4 v[QUANT_NV];
+        if (q.vec) {
+            quant_load<TRANS, true>(v, q.src, q.lds, q.rows, q.cols, ti * 128, tj * 128);
+            quant_tile<TRANS, true>(v, q.rows, q.cols, q.width, ti * 128, tj * 128, d, (int)ldd, so, 1, red, tile,
+                                    [] {});
+        } else {
+            quant_load<TRANS, false>(v, q.src, q.lds, q.rows, q.cols, ti * 128, tj * 128);
+            quant_tile<TRANS, false>(v, q.rows, q.cols, q.width, ti * 128, tj * 128, d, (int)ldd, so, 1, red, tile,
+                                     [] {});
+        }
         __syncthreads();   // red is reused by the next item
     }
     pdl_trigger();
@@ -497,7 +607,14 @@ static bool quant_op(QuantOp* o, int rows, int cols, const float* src, int lds, 
 }
 
 static pgk_status launch_quant_ops(const QuantOp& a, const QuantOp& b, cudaStream_t st) {
-    PGK_CUDA_TRY(launch_pdl(k_quant_fp8, (unsigned)a.items + (unsigned)b.items, QUANT_THREADS, 0, 1, st, a, b),
+    static SmemLimit limit;
+    PGK_CUDA_TRY(allow_smem(limit, (const void*)k_quant_fp8, QUANT_STAGE_BYTES), "FP8 quantisation set-up");
+    pgk_machine m;
+    const unsigned items = (unsigned)a.items + (unsigned)b.items;
+    const bool prefetch = (a.items == 0 || a.vec_in) && (b.items == 0 || b.vec_in) &&
+                          current_machine(&m, NULL) == PGK_OK && items > 2u * (unsigned)m.sm_count;
+    PGK_CUDA_TRY(launch_pdl(k_quant_fp8, prefetch ? 2u * (unsigned)m.sm_count : items, QUANT_THREADS,
+                            prefetch ? QUANT_STAGE_BYTES : 0, 1, st, a, b),
                  "FP8 quantisation launch");
     return PGK_OK;
 }

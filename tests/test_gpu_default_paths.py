@@ -209,7 +209,7 @@ def test_skinny_products_over_k_ranges(dev, form, M, N, K, pad, beta):
     assert torch.isnan(C[:, N:]).all()
 
 
-@pytest.mark.parametrize("R,Cc", [(128, 128), (5, 300), (257, 131), (640, 384)])
+@pytest.mark.parametrize("R,Cc", [(128, 128), (5, 300), (257, 131), (640, 384), (2601, 2502)])
 @pytest.mark.parametrize("kind", ["ties", "tiny", "huge", "specials"])
 def test_fp8_codes_bit_exact_on_hard_tiles(dev, R, Cc, kind):
     """Tiles whose quotients lie on or beside the midpoints of E4M3, scales too small or too
@@ -240,3 +240,18 @@ def test_fp8_codes_bit_exact_on_hard_tiles(dev, R, Cc, kind):
         qt = torch.zeros(Cc, (R + 15) // 16 * 16, dtype=torch.uint8, device=dev)
         pgk.quant_fp8(W[:, :Cc], qt, s, 1)
         assert np.array_equal(qt.cpu().numpy()[:, :R], codes.T)
+
+
+@pytest.mark.parametrize("pad_a,pad_b", [(0, 1), (1, 0), (1, 1)])
+def test_fp8_operands_of_different_alignment_in_one_launch(dev, pad_a, pad_b):
+    """Blocks that take several tiles, of either operand, with and without 128-bit loads: the
+    same product bit by bit as with both operands on 16-byte rows."""
+    M, N, K = 2561, 2600, 2500
+    A, B = (torch.from_numpy(x).to(dev) for x in inputs.gemm_operands(M, N, K, seed=9))
+    ref = torch.empty(M, N, device=dev)
+    pgk.gemm(A, B, ref, pgk.FP8_E4M3, None)
+    Ap, Bp = torch.zeros(M, K + pad_a, device=dev), torch.zeros(K, N + pad_b, device=dev)
+    Ap[:, :K], Bp[:, :N] = A, B
+    C = torch.empty(M, N, device=dev)
+    pgk.gemm(Ap[:, :K], Bp[:, :N], C, pgk.FP8_E4M3, None)
+    assert torch.equal(C, ref)
