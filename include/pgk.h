@@ -111,9 +111,12 @@ typedef struct {
  *    multiple of 4 (else ALIGNMENT).  sr >= 2 splits K into sr slices (work
  *    units: 128-row tile x slice) whose partial products a second launch sums
  *    in slice order (deterministic; a library workspace holds sr x M x N
- *    floats); sr = 1: one slice; sr = 0: as many slices as fill the SMs when
- *    the row tiles alone do not, each at least 512 deep.  pgk_gemm without
- *    parameters takes (128, 64, s, 0) for N <= 64 when A qualifies. */
+ *    floats); sr = 1: one slice; sr = 0: the K blocks of all row tiles cut into
+ *    one contiguous range per SM, each at least 512 deep, where that beats whole
+ *    tiles; a second launch adds the pieces of shared tiles in range order
+ *    (workspace: 256 x N floats per range; without it the tiles run whole).
+ *    pgk_gemm without parameters takes (128, 64, s, 0) for N <= 64 when A
+ *    qualifies. */
 typedef struct { int B0, B1, s, sr, tile; } pgk_params;
 
 /* Leaves of the case discussion, with the paper's labels (Section 5):
@@ -219,8 +222,8 @@ PGK_API pgk_status pgk_select_case_regs(const pgk_machine* machine, const int* r
 /* C = A*B (beta = 0) or C += A*B (beta = 1, the accumulate form c += a*b of
  * Fig. "metamul").  A, B, C are FP32 device matrices (row-major, see top).
  * `dtype` selects the arithmetic form (pgk_dtype).  `prog` = NULL uses the
- * tuned parameters cached for (device, M, N, K, dtype) by pgk_autotune, else a
- * default; otherwise the case discussion runs on `prog` for the current
+ * tuned parameters cached for (device, M, N, K, dtype) by pgk_autotune, else
+ * plans tiles and K slices by the shape; otherwise the case discussion runs on `prog` for the current
  * device's machine parameters.  Tensor-core forms convert A and B into library
  * workspaces first (pgk_cvt_bf16 / pgk_split_bf16 / pgk_quant_fp8).
  * Errors: INVALID_ARG, INFEASIBLE, UNSUPPORTED, CUDA, NO_MEMORY. */
@@ -274,7 +277,8 @@ PGK_API pgk_status pgk_gemm_case(const pgk_case* c, int M, int N, int K, const f
  * `problems`, device matrix pointers) and the tile prefix sums into a device
  * table; every CTA pulls (problem, tile) work items from an atomic counter
  * until all tiles are done.  `prog` selects the register-blocked tile variant
- * (NULL = tuned/default).  use_graph = 1 captures the counter reset and the
+ * (NULL = tuned, else single-warp 64 x 64 tiles with K slices by the amount of
+ * work).  use_graph = 1 captures the counter reset and the
  * launch in a CUDA graph, cached per problem set and replayed on later calls
  * with the same problems.
  * PGK_BF16 / PGK_SPLIT_BF16 / PGK_FP8_E4M3: the operands are converted into

@@ -2268,9 +2268,9 @@ static pgk_status tc_gemm_fused(const TcVariant& v, int slices, int M, int N, in
                 stream = false;
             }
         }
-        if (stream) {
-            p.part = (float*)workspace(WS_SPLITK, 2 * G * piece, &st);
-            if (!p.part) return st;
+        // (without the workspace the tiles run whole)
+        if (stream) p.part = (float*)workspace(WS_SPLITK, 2 * G * piece, &st);
+        if (stream && p.part) {
             p.stream = G;
             cudaError_t e = v.launch(maps, p, G, m.sm_count, s);
             if (e != cudaSuccess) return cuda_fail(e, "fused-conversion GEMM launch");
