@@ -569,7 +569,7 @@ def roofline(form, alg, gemm_ms, step_ms, machine, pk, pk_src, clocks, traffic=N
         peak = machine.sm_count * 128 * 2 * f * 1e6 / 1e12
         out = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                "frac": achieved / peak, "traffic": traffic,
-               "kernel": "k_rb (register-blocked FP32 SIMT)",
+               "kernel": "k_wt or k_rb (register-tiled FP32 SIMT)",
                "peak_source": f"{machine.sm_count} SMs x 128 FP32 lanes x 2 flop x {f:.0f} MHz "
                               f"(max SM clock, {pk_src})"}
         if clocks.get("sm_mhz"):
