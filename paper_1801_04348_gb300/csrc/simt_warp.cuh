@@ -63,11 +63,17 @@ __device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, int by
 // VA, VB: A (or B) is read 16 bytes at a time, which needs its base and row stride on
 // 16-byte boundaries and K (or N) a multiple of 4 (a float4 then lies wholly inside or
 // outside the matrix); otherwise by 4-byte asynchronous copies, lanes along the rows (along
-// K, and transposed into place without bank conflicts, for A).  Rows and columns beyond M
-// and N are read at the last row or column instead (their outputs are never stored), K
-// beyond its end reads as zero.
+// K, and transposed into place without bank conflicts, for A).  K beyond its end reads as
+// zero.  Rows and columns beyond M and N are copied from others (their outputs are never
+// stored): from distinct ones, because lanes that copy the same word, as when all read the
+// last column, are served one after the other, and the edge tiles then held up the launch
+// (605 x 773 x 1491, 130 tiles, 90 -> 42 us; 434 x 263 x 1560 38 -> 19).
 template <class Cfg, bool VA, bool VB>
 struct WarpTile {
+    // x where it is below n, else a value below it, distinct for neighbouring x; mask: the
+    // largest power of two up to n, less one (multiples of 4 stay multiples of 4)
+    static __device__ __forceinline__ int inside(int x, int n, int mask) { return x < n ? x : x & mask; }
+
     static __device__ __forceinline__ void sync() {
         if (Cfg::NW == 1) __syncwarp();
         else __syncthreads();
@@ -94,6 +100,7 @@ struct WarpTile {
         constexpr int AM_STEP = Cfg::NT / (BK / 4), BK_STEP = Cfg::NT / (Cfg::BN / 4);
         static_assert(Cfg::NT % (BK / 4) == 0 && Cfg::NT % (Cfg::BN / 4) == 0, "fixed column per thread");
 
+        const int mask_m = (int)(0x7fffffffu >> __clz(M)), mask_n = (int)(0x7fffffffu >> __clz(N));
         auto load_a = [&](int k0, int buf) {
             if (VA) {
                 const int gk = k0 + 4 * akq;
@@ -111,7 +118,7 @@ struct WarpTile {
 #pragma unroll
                 for (int i = 0; i < 4 * Cfg::LA; ++i)
                     cp_async4(d + 4u * (uint32_t)(i * (Cfg::NT / BK)),
-                              p + (size_t)min(row0 + m + i * (Cfg::NT / BK), M - 1) * lda, in ? 4 : 0);
+                              p + (size_t)inside(row0 + m + i * (Cfg::NT / BK), M, mask_m) * lda, in ? 4 : 0);
             }
         };
         auto store_a = [&](int buf) {
@@ -129,7 +136,7 @@ struct WarpTile {
         auto load_b = [&](int k0, int buf) {   // (closes the group of copies of A, too)
             const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(Bs + buf * Cfg::B_ELEMS);
             if (VB) {
-                const int gn = min(col0 + 4 * bnq, N - 4);
+                const int gn = inside(col0 + 4 * bnq, N, mask_n);
 #pragma unroll
                 for (int i = 0; i < Cfg::LB; ++i) {
                     const int k = bk + i * BK_STEP;
@@ -144,7 +151,7 @@ struct WarpTile {
                     const int e = tid + i * Cfg::NT, k = e / Cfg::BN, n = e % Cfg::BN;
                     const bool in = k0 + k < k_end;
                     cp_async4(d0 + 4u * (uint32_t)(k * Cfg::LDBS + n),
-                              B + (size_t)(in ? k0 + k : 0) * ldb + min(col0 + n, N - 1), in ? 4 : 0);
+                              B + (size_t)(in ? k0 + k : 0) * ldb + inside(col0 + n, N, mask_n), in ? 4 : 0);
                 }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
