@@ -262,25 +262,22 @@ static const GroupedVariant* find_grouped(const pgk_params* prog) {
 
 // The variant of a group without parameters: 64 x 64 tiles with as many K slices (warps) as
 // give the smallest estimate: the work spread over the SMs' eight warps each, or the longest
-// tile if that is more, and half a longest tile for the uneven end.  A K step of a tile costs a warp 304 cycles beside a second one on its scheduler, a
-// tile 6000 more (its problem, first loads and stores), and K slices meet at 256 cycles each.
-// Measured: 512 problems up to 2048 a side take one slice, 1.97 ms (64 x 64 tiles of 256
-// threads: 4.05); ten of them, 823 tiles, 72 us (one slice 345, 256 threads 145).  Where most of the work reads unaligned rows and there
-// are tiles for every warp, the 128 x 64 tiles of 128 threads are faster (512 problems of odd
-// sizes: 2.59 ms against 3.55): they copy half as many elements per product.
+// tile if that is more, and half a longest tile for the uneven end.  A K step of a tile costs
+// a warp 304 cycles beside a second one on its scheduler, a tile 6000 more (its problem, first
+// loads and stores), and K slices meet at 256 cycles each.  Measured: 512 problems up to 2048
+// a side take one slice, 1.95 ms (64 x 64 tiles of 256 threads: 4.05); ten of them, 823 tiles,
+// 72 us (one slice 345, 256 threads 145).  Unaligned problems take the same tiles: 300 of odd
+// sizes up to 900 take 1.33 ms and 1.46 in 128 x 64 tiles of 128 threads, 512 up to 300 0.161
+// and 0.171.
 static const GroupedVariant* grouped_default(int G, const pgk_problem* pr, int sms) {
     static const GroupedVariant t[] = {gv_wt<1>(), gv_wt<2>(), gv_wt<4>(), gv_wt<8>()};
-    double tiles = 0, steps = 0, unaligned = 0, longest = 0;
+    double tiles = 0, steps = 0, longest = 0;
     for (int i = 0; i < G; ++i) {
         const double n = (double)((pr[i].M + 63LL) / 64) * (double)((pr[i].N + 63LL) / 64);
         tiles += n;
         steps += n * pr[i].K;
-        if (!al16(pr[i].A) || !al16(pr[i].B) || pr[i].lda % 4 || pr[i].ldb % 4 || pr[i].K % 4 || pr[i].N % 4)
-            unaligned += n * pr[i].K;
         longest = std::max(longest, (double)pr[i].K);
     }
-    const pgk_params wide = {16, 8, 8, 8, 8};
-    if (2 * unaligned > steps && tiles >= 8.0 * sms) return find_grouped(&wide);
     const GroupedVariant* best = &t[0];
     double best_t = 0;
     for (const GroupedVariant& v : t) {
