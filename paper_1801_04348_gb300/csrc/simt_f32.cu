@@ -281,9 +281,8 @@ struct WtPlan {
 // slices), 2048^3 in 283 (331 with 128 x 128 tiles, 256 of them on 304 places).
 // Rows of C off the 16-byte boundaries are written 4 bytes a lane, and the warps of a 128 x
 // 128 tile do so at once where eight single-warp tiles take turns: 2000 cycles a block more.
-// 4384 x 1565 x 48 takes 24.7 us in 64 x 64 tiles and 28.3 in 128 x 128 ones, 3417 x 2576 x
-// 609 takes 264 and 246.  K slices of a 64 x 64 tile, which meet before the store, cost 1000:
-// 2974 x 321 x 112 takes 18.2 us in two of them and 14.5 in 32 x 32 tiles.
+// 4384 x 1565 x 48 takes 24.7 us in 64 x 64 tiles and 27.3 in 128 x 128 ones, 3417 x 2576 x
+// 609 takes 235 and 224.
 // More than one group needs a workspace, shared per device, which short products never
 // used: it is limited to K >= 4096 with few tiles, where every program splits K, and left
 // out while the stream is being captured (a workspace cannot grow there).
@@ -304,8 +303,7 @@ static WtPlan wt_plan(const SimtArgs& p, int sms, bool groups_allowed, int tile)
             const double resident = k.tile == 32 ? 4 : 2;   // warps per scheduler (registers)
             double t = steps * (per_sched <= 1 ? k.alone : k.shared * per_sched) +
                        2000 * ceil(per_sched / resident);
-            if (!p.vecC && (k.tile == 128 || (k.tile == 64 && k.ks > 1)))
-                t += (k.tile == 128 ? 2000 : 1000) * blocks;
+            if (k.tile == 128 && !p.vecC) t += 2000 * blocks;
             if (k.ks > 1) t += blocks * (k.ks * k.tile * k.tile / 16 + 300);
             if (g > 1) t += 9000 + (double)g * M * N * 8 / 3400;
             if (!best.kind || t < best_t) {
